@@ -262,6 +262,7 @@ inline int sm_count() {
 }
 
 constexpr int TILE = 128;          // particles per tile (= threads per block)
+constexpr int ENTRY_PAD = 16;       // entries past the end that the list search may read
 constexpr int MAX_TYPES = ESPP_MAX_TYPES;
 
 }  // namespace espp

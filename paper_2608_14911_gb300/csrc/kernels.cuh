@@ -85,10 +85,10 @@ template <class T> struct DevSys {
     // compact entries (position, storage slot in the w lane): those of cell h
     // are cell_ent[cell_beg[h] .. cell_beg[h + 1]), ascending slot
     V4<T>* cell_ent;
+    float4* cell_ent32;     // FP64 handles: the entries' coordinates in FP32 (list search)
     int* cell_beg;          // ncells + 1; cell_beg[ncells] = N
     int* rank_start;        // first new slot of each cell in Hilbert-rank order (resort only)
     int cell_w;             // cell subdivision: cells of edge >= (rc + skin) / cell_w (1, 2 or 3)
-    int list_push;          // Verlet build: hits pushed into the list group (1) or placed (0)
     const int* cell_by_rank;  // global Hilbert rank -> cell index
     const int* cell_rep;
     int ncells;
@@ -230,6 +230,18 @@ __device__ __forceinline__ void le_wrap(double p[3], double& vx, int k[3], const
     }
 }
 
+// cell index along one edge of a coordinate inside the box
+template <class T>
+__device__ __forceinline__ int cell_coord(T x, T cpl, int nc) {
+    int c = (int)(x * cpl);
+    c = c < 0 ? 0 : c;
+    return c >= nc ? nc - 1 : c;
+}
+
+// the cell entries in FP32, as the list search reads them
+__device__ __forceinline__ const float4* entries_f(const DevSys<float>& s) { return s.cell_ent; }
+__device__ __forceinline__ const float4* entries_f(const DevSys<double>& s) { return s.cell_ent32; }
+
 // kernels launched by one rebuild without a resort (Launch::rebuild)
 constexpr int REBUILD_LAUNCHES = 8;
 
@@ -246,6 +258,8 @@ template <class T> struct Launch {
     // rebuild pipeline on the positions in buffer `cur` (other buffer is
     // scratch); returns the number of kernels launched
     static int rebuild(const DevSys<T>& s, int cur, bool resort, bool permute_force, cudaStream_t st);
+    // the list search of the replicas just binned (k_verlet.cu)
+    static void verlet(const DevSys<T>& s, cudaStream_t st);
     static void request_all(const DevSys<T>& s, cudaStream_t st);
     // step kernels
     // one force evaluation (+ the learned potential's kernels); returns the

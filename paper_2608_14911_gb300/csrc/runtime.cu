@@ -313,7 +313,8 @@ class System : public SystemBase {
             (rc = alloc(&d.frc, n, allocs)) || (rc = alloc(&d.frc_alt, n, allocs)) ||
             (rc = alloc(&d.xb, n, allocs)) || (rc = alloc(&d.img, n, allocs)) ||
             (rc = alloc(&d.img_alt, n, allocs)) || (rc = alloc(&d.bond_slot, n, allocs)) ||
-            (rc = alloc(&d.cell_ent, n, allocs)))
+            (rc = alloc(&d.cell_ent, n + ENTRY_PAD, allocs)) ||
+            (sizeof(T) == 8 && (rc = alloc(&d.cell_ent32, n + ENTRY_PAD, allocs))))
             return rc;
         int2* bg = nullptr;
         int *sid, *perm, *cellh, *inc, *ncnt, *req, *now, *rto;
@@ -1891,15 +1892,14 @@ class System : public SystemBase {
         const int method_of[NSH] = {ESPP_FORCES_VERLET, ESPP_FORCES_VERLET, ESPP_FORCES_VERLET,
                                     ESPP_FORCES_CELLS,  ESPP_FORCES_VERLET, ESPP_FORCES_VERLET};
         const int w_of[NSH] = {1, 2, 3, 1, 1, 3};
-        const int push_of[NSH] = {0, 0, 0, 0, 1, 1};
+        // shapes 4 and 5 name shapes 0 and 2 (one list store serves both)
+        const int same_as[NSH] = {0, 1, 2, 3, 0, 2};
         auto apply = [&](int k) -> int {
-            // the subdivision and the list store first (the list-free shape
-            // takes whole cells), then the method (a change of method
-            // rebuilds the grid)
+            // the subdivision first (the list-free shape takes whole cells),
+            // then the method (a change of method rebuilds the grid)
             cell_sub_req = w_of[k];
-            int rc = set_list_store(push_of[k]);
+            const int rc = set_force_method(method_of[k]);
             if (rc) return rc;
-            if ((rc = set_force_method(method_of[k]))) return rc;
             return build_neighbors(rc_list, skin);
         };
         double t[NSH];
@@ -1909,6 +1909,10 @@ class System : public SystemBase {
         CK(cudaEventCreate(&e1));
         for (int k = 0; k < NSH && !rcode; ++k) {
             if (method_of[k] == ESPP_FORCES_CELLS && d.mlp_on) continue;
+            if (same_as[k] != k) {
+                t[k] = t[same_as[k]];
+                continue;
+            }
             const int rc = apply(k);
             if (rc == ESPP_ERR_BOX_TOO_SMALL) continue;  // this shape does not fit
             if ((rcode = rc) || (rcode = restore()) || (rcode = integrate(2, dt, gamma, kT))) break;
@@ -2053,8 +2057,6 @@ class System : public SystemBase {
     int set_list_store(int push) override {
         if (push != ESPP_LIST_STORE_PLACE && push != ESPP_LIST_STORE_PUSH)
             return fail(ESPP_ERR_ARG, "unknown list store");
-        d.list_push = push;
-        clear_graphs();  // a kernel argument of the captured graphs
         return ESPP_OK;
     }
 

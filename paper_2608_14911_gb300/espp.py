@@ -497,9 +497,9 @@ class System:
 
     def tune_force_method(self, nsteps, dt, gamma, kT):
         """Time the FORCE_SHAPES shapes (Verlet over whole, half or third
-        cells, list-free cells, whole and third cells with pushed list
-        stores) from the current state and keep the fastest; returns (ms per
-        step of each, chosen shape index)."""
+        cells, list-free cells, then whole and third cells again under their
+        second names) from the current state and keep the fastest; returns
+        (ms per step of each, chosen shape index)."""
         ms = (ctypes.c_double * FORCE_SHAPES)()
         ch = ctypes.c_int32()
         self._c(lib().espp_tune_force_method(self._h, int(nsteps), float(dt), float(gamma), float(kT), ms,

@@ -1,0 +1,94 @@
+"""The Verlet list search at the sizes where it can go wrong: boxes of the
+fewest cells (every row wraps), long flat boxes, rows and lists longer than a
+lane's buffer, both forms of the search (one thread or a team of lanes per
+particle) and particle counts at the tile edges.  The neighbour sets are the
+oracle's brute-force ones, FP32 outside a band of 1e-6 sigma at the list radius
+(the rounding of coordinates up to a few tens of sigma), FP64 exactly."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2608_14911_gb300 import espp, inputs as I
+
+pytestmark = pytest.mark.gpu
+FP32, FP64 = espp.ESPP_FP32, espp.ESPP_FP64
+RL = 1.5
+
+
+def _gas(n, box, seed, blob=0):
+    """n uniform positions, the first `blob` of them in a ball of radius 0.9."""
+    c = I.random_positions(n, box, seed=seed)
+    g = np.random.default_rng(seed)
+    if blob:
+        d = g.normal(size=(blob, 3))
+        d *= 0.9 * g.random((blob, 1)) ** (1 / 3) / np.linalg.norm(d, axis=1, keepdims=True)
+        c.x[:blob] = I.f32(np.mod(0.25 + d, c.box))
+        c.x[c.x >= c.box] = 0.0
+    return c
+
+
+def _handle(c, prec, w):
+    s = espp.System(c.box, c.n, c.types, c.bonds, precision=prec, seed=3)
+    s.set_lj_capped(1.0, 1.0, 1.1, 0.8)
+    s.set_cell_subdivision(w)
+    s.set_state(c.x, None, c.img)
+    s.build_neighbors(1.1, RL - 1.1)
+    return s
+
+
+@pytest.mark.parametrize("prec", [FP32, FP64])
+@pytest.mark.parametrize("w", [1, 2, 3])
+@pytest.mark.parametrize("n,box,blob", [
+    (1, (4.6, 4.6, 4.6), 0),
+    (129, (4.6, 4.7, 4.8), 0),             # the fewest cells: every row crosses a face
+    (1500, (40.0, 4.6, 5.3), 0),           # long rows along x
+    (2000, (5.0, 4.6, 60.0), 0),
+    (900, (9.0, 8.0, 7.7), 140),           # lists longer than a lane's buffer, around a corner
+    (8191, (22.0, 20.0, 21.0), 60),        # the team form's last size (FP32)
+    (8192, (22.0, 20.0, 21.0), 60),
+])
+def test_neighbour_sets(prec, w, n, box, blob):
+    c = _gas(n, box, 11 + n, blob)
+    s = _handle(c, prec, w)
+    row, cols = s.get_neighbors()
+    s.close()
+    orow, ocols = O.neighbors(c.box, c.x, RL, method="brute")
+    band = 1e-6 if prec == FP32 else 0.0
+    for i in range(c.n):
+        got = cols[row[i]:row[i + 1]].tolist()
+        assert len(set(got)) == len(got)
+        for j in set(got) ^ set(ocols[orow[i]:orow[i + 1]].tolist()):
+            d = c.x[i] - c.x[j]
+            d -= c.box * np.round(d / c.box)
+            assert abs(np.linalg.norm(d) - RL) <= band, (i, j)
+
+
+@pytest.mark.parametrize("prec,n", [(FP32, 5000), (FP64, 20000)])
+def test_both_forms_build_the_same_lists(prec, n):
+    # two replicas together are past the size up to which a team of lanes
+    # shares a particle, each alone is below it: the same forces and
+    # trajectories (rebuilds included) bit for bit
+    cs = [_gas(n, (19.0 * (n / 5000) ** (1 / 3),) * 3, seed) for seed in (5, 6)]
+    alone = []
+    for c in cs:
+        s = _handle(c, prec, 1)
+        f = s.compute_forces()
+        s.integrate(25, 0.002, 1.0, 1.0)
+        alone.append((f, s.get_state()))
+        assert s.n_rebuilds >= 2
+        s.close()
+    b = espp.System(precision=prec, replicas=[dict(box=c.box, n=c.n, types=c.types, bonds=c.bonds, seed=3)
+                                              for c in cs])
+    b.set_lj_capped(1.0, 1.0, 1.1, 0.8)
+    b.set_cell_subdivision(1)
+    b.set_state(np.concatenate([c.x for c in cs]), None, np.concatenate([c.img for c in cs]))
+    b.build_neighbors(1.1, RL - 1.1)
+    fb = b.compute_forces()
+    b.integrate(25, 0.002, 1.0, 1.0)
+    st = b.get_state()
+    b.close()
+    for k, (f, q) in enumerate(alone):
+        sl = slice(k * n, (k + 1) * n)
+        assert np.array_equal(f, fb[sl])
+        for a, p in zip(q, st):
+            assert np.array_equal(a, p[sl])
