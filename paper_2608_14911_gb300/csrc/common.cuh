@@ -81,6 +81,35 @@ __device__ __forceinline__ T drift(T x, T v, T dt) {
 }
 
 // ---------------------------------------------------------------------------
+// Comparisons that keep FP64 off its unit (a double compare occupies it like an
+// addition; GB300 has two FP64 lanes per SM): non-negative doubles order as
+// their bit patterns, a NaN compares false as it does in floating point.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ bool less_nonneg(float a, float b) { return a < b; }
+__device__ __forceinline__ bool less_nonneg(double a, double b) {
+    return (unsigned long long)__double_as_longlong(a) < (unsigned long long)__double_as_longlong(b);
+}
+// |a| > b for b >= 0 (a NaN counts as larger)
+__device__ __forceinline__ bool abs_greater(float a, float b) { return fabsf(a) > b; }
+__device__ __forceinline__ bool abs_greater(double a, double b) {
+    return (unsigned long long)(__double_as_longlong(a) & 0x7fffffffffffffffll) >
+           (unsigned long long)__double_as_longlong(b);
+}
+// |a| < b for b > 0 (false for a NaN)
+__device__ __forceinline__ bool abs_less(float a, float b) { return fabsf(a) < b; }
+__device__ __forceinline__ bool abs_less(double a, double b) {
+    return (unsigned long long)(__double_as_longlong(a) & 0x7fffffffffffffffll) <
+           (unsigned long long)__double_as_longlong(b);
+}
+// a > 0 (false for a NaN)
+__device__ __forceinline__ bool positive(float a) { return a > 0.f; }
+__device__ __forceinline__ bool positive(double a) {
+    return (unsigned long long)(__double_as_longlong(a) - 1) < 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool negative(float a) { return a < 0.f; }
+__device__ __forceinline__ bool negative(double a) { return __double2hiint(a) < 0; }
+
+// ---------------------------------------------------------------------------
 // Minimum image of xi - xj for coordinates stored in [0, L).  The periodic
 // shift is applied to the larger coordinate first; that subtraction is exact
 // (Sterbenz: the coordinate lies in [L/2, L)), so the result carries a single
@@ -88,10 +117,9 @@ __device__ __forceinline__ T drift(T x, T v, T dt) {
 // ---------------------------------------------------------------------------
 template <class T>
 __device__ __forceinline__ T min_image(T xi, T xj, T L, T halfL) {
-    T d = xi - xj;
-    if (d > halfL) d = (xi - L) - xj;
-    else if (d < -halfL) d = xi - (xj - L);
-    return d;
+    const T d = xi - xj;
+    if (!abs_greater(d, halfL)) return d;
+    return negative(d) ? xi - (xj - L) : (xi - L) - xj;
 }
 
 // ---------------------------------------------------------------------------

@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(256) k_cellsort(DevSys<T> s) {
         if constexpr (sizeof(T) == 8)
             for (int k = 0; k < e; ++k) {
                 const V4<T> q = p[k];
-                s.cell_ent32[s.cell_beg[h] + k] = make_float4((float)q.x, (float)q.y, (float)q.z, 0.f);
+                s.cell_ent32[s.cell_beg[h] + k] = make_float4((float)q.x, (float)q.y, (float)q.z, __int_as_float(bits_as_int(q.w)));
             }
         // list-free mode with DPD: the velocities in entry order as well
         if (s.cells_mode && s.dpd)
@@ -244,6 +244,7 @@ __global__ void __launch_bounds__(256) k_resort_scatter(DevSys<T> s) {
         for (int k = 0; k < e; ++k) {
             s.perm[b + k] = bits_as_int(p[k].w);
             p[k].w = int_bits_as(T(0), b + k);
+            if constexpr (sizeof(T) == 8) s.cell_ent32[s.cell_beg[c] + k].w = __int_as_float(b + k);
         }
     }
 }
@@ -320,7 +321,7 @@ int Launch<T>::rebuild(const DevSys<T>& s, int cur, bool resort, bool permute_fo
     }
     // list-free mode: the binning is all that is needed
     if (s.cells_mode) return launched;
-    Launch<T>::verlet(s, st);
+    Launch<T>::verlet(s, cur, st);
     launched += 1;
     // mirrored entries for the learned potential's pair-once evaluation
     if (s.mlp_on && s.mlp_rev) launched += Launch<T>::mlp_rev(s, st);

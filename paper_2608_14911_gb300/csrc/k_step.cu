@@ -38,7 +38,7 @@ constexpr StepShape STEP_SHAPES[ESPP_STEP_SHAPES] = {{1, 8, 1}, {2, 8, 1}, {1, 1
 #define ESPP_STEP_MINB32 8  // KG 1M FP32: 0.1027 ms per step (8), 0.1123 (10)
 #endif
 #ifndef ESPP_STEP_MINB32_DPD  // the same for the DPD variants
-#define ESPP_STEP_MINB32_DPD 10
+#define ESPP_STEP_MINB32_DPD 7
 #endif
 #ifndef ESPP_STEP_LATE  // loads issued after the pair loop: 1 bond partners, 2 velocity and build position
 #define ESPP_STEP_LATE 3  // KG 1M FP32 at 8 blocks per SM: 58.7 us (3), 61.5 (1); fewer values live across the loop
@@ -53,17 +53,16 @@ namespace espp {
 // read in batches of int4 groups: all indices of a batch first, then all
 // neighbour positions, then the arithmetic, so that each thread keeps several
 // independent loads in flight; the next batch's indices are prefetched.
-// With DPD the thermostat's pair term is added in the same pass, for pairs
-// inside the DPD cutoff, from the neighbours' velocity snapshot.
+// (FP32 without DPD; FP64 handles and the DPD thermostat take queue_loop.)
 // Entries with x code 3 cross a sheared face (Lees-Edwards): their x
 // difference is taken from the current offset in *le.
-template <class T, bool ENERGY, bool MULTI, bool FAST, bool DPD, bool LE, int GB32 = 1>
+template <class T, bool ENERGY, bool MULTI, bool FAST, bool LE, int GB32 = 1>
 __device__ __forceinline__ void pair_loop(const DevSys<T>& s, const V4<T>* __restrict__ P, int i, int n,
                                           const V4<T>& xi, int ti, const PairRec<T>* pr1,
                                           T L0, T L1, T L2, T& fx, T& fy, T& fz, T& pe, T& vir, T& vxz,
-                                          const LeCtx<T>* le, const DpdCtx<T>* dc = nullptr) {
+                                          const LeCtx<T>* le) {
     const T xim = xi.x - L0, yim = xi.y - L1, zim = xi.z - L2;
-    constexpr int GB = sizeof(T) == 4 ? GB32 : 1;  // int4 groups per batch
+    constexpr int GB = GB32;  // int4 groups per batch
     const int ng = (n + 3) >> 2;
     const int4* __restrict__ nb = reinterpret_cast<const int4*>(s.nbr) + i;
     const size_t stride = (size_t)s.stride;
@@ -79,7 +78,7 @@ __device__ __forceinline__ void pair_loop(const DevSys<T>& s, const V4<T>* __res
     const int4 pad4 = make_int4(pad, pad, pad, pad);
     // FP32 single-type Lennard-Jones without energies (the step's hot path):
     // two entries per packed FP32x2 instruction, forces summed in two lanes
-    constexpr bool PACK = sizeof(T) == 4 && FAST && !ENERGY && !DPD;
+    constexpr bool PACK = FAST && !ENERGY;
     f32x2 px = 0ull, py = 0ull, pz = 0ull;
     f32x2 xi2 = 0ull, yi2 = 0ull, zi2 = 0ull, sg2 = 0ull, e24 = 0ull;
     if constexpr (PACK) {
@@ -167,34 +166,20 @@ __device__ __forceinline__ void pair_loop(const DevSys<T>& s, const V4<T>* __res
                 const T dx = xi.x - xj[q].x, dy = xi.y - xj[q].y, dz = xi.z - xj[q].z;
                 pair_term<T, ENERGY, MULTI, FAST>(s, ti, pr1, dx, dy, dz, bits_as_int(xj[q].w), fx, fy, fz, pe,
                                                   vir, vxz);
-                if (DPD) {
-                    const T r2 = dx * dx + dy * dy + dz * dz;
-                    if (r2 < s.ip->dpd_rc2)
-                        dpd_term<T>(s.ip, *dc, dx, dy, dz, r2, ld4<T>(s.vsnap + nbr_slot(jj[q])), fx, fy, fz);
-                }
             }
         } else {
 #pragma unroll
             for (int q = 0; q < 4 * GB; ++q) {
                 const int code = nbr_code(jj[q]);
-                int nz = 0;
                 T dx;
-                if (LE && (code & 3) == 3) {
-                    nz = (code >> 4) == 1 ? 1 : -1;
-                    dx = le_dx(xi.x, xj[q].x, nz, le->d, L0, le->inv_Lx);
-                } else {
+                if (LE && (code & 3) == 3)
+                    dx = le_dx(xi.x, xj[q].x, (code >> 4) == 1 ? 1 : -1, le->d, L0, le->inv_Lx);
+                else
                     dx = shifted_diff(xi.x, xim, xj[q].x, L0, code & 3);
-                }
                 const T dy = shifted_diff(xi.y, yim, xj[q].y, L1, (code >> 2) & 3);
                 const T dz = shifted_diff(xi.z, zim, xj[q].z, L2, code >> 4);
                 pair_term<T, ENERGY, MULTI, FAST>(s, ti, pr1, dx, dy, dz, bits_as_int(xj[q].w), fx, fy, fz,
                                                   pe, vir, vxz);
-                if (DPD) {
-                    const T r2 = dx * dx + dy * dy + dz * dz;
-                    if (r2 < s.ip->dpd_rc2)
-                        dpd_term<T>(s.ip, *dc, dx, dy, dz, r2, ld4<T>(s.vsnap + nbr_slot(jj[q])), fx, fy, fz,
-                                    nz);
-                }
             }
         }
     }
@@ -206,6 +191,214 @@ __device__ __forceinline__ void pair_loop(const DevSys<T>& s, const V4<T>* __res
         fy += a + b;
         f2split(pz, a, b);
         fz += a + b;
+    }
+}
+
+// ---- the warp's pair queue ---------------------------------------------------
+// FP64 handles and the DPD thermostat: a pair's term is expensive (FP64
+// instructions at a small fraction of the FP32 rate; a Philox block) and a
+// quarter to two thirds of the list entries lie beyond the cutoff, so a thread
+// that walks its own list runs the term for nearly every entry, with the lanes
+// whose entry is inside.  Here a warp first tests QG groups of every list in
+// FP32 (FP64 handles: on coordinates cut to FP32, against a widened cutoff) and
+// keeps the entries inside, then evaluates the warp's entries 32 at a time, one
+// per lane whoever owns them, the exact test included, into shared memory; every
+// particle then adds its own terms in list order, as a walk of the list would.
+// Step kernel, walking its own list / queue: KG melt of 1M FP64 876 / 464 us, LJ
+// fluid of 256,000 FP64 1241 / 822 us, DPD fluid of 786,432 FP32 446 / 323 us (215 M
+// warp instructions instead of 284 M, 26 of 32 lanes active instead of 11).
+template <class T, bool DPD, int PPW>
+struct PairQueue {
+    // list groups per block of the queue, terms held at a time.  FP32: small,
+    // for the shared memory they take is L1 that the gathers lose (DPD fluid of
+    // 786,432, step kernel: 4 / 128 320 us, 8 / 256 552 us, 4 / 64 329 us); FP64:
+    // large, for every stretch of terms costs its particles' additions once
+    // more (KG melt of 1M: 8 / 256 530 us, 4 / 128 570 us, 4 / 64 609 us)
+    static constexpr int QG = sizeof(T) == 8 ? 8 : 4;
+    static constexpr int QR = sizeof(T) == 8 && !DPD ? 256 : 128;
+    int col[QG * 4 * PPW];  // entries inside: row k of the particle's column
+    T fr[QR], dx[QR], dy[QR], dz[QR];
+    T th[DPD ? QR : 1];     // the thermostat's term
+};
+
+// a coordinate in FP32: FP64 ones are cut to 20 mantissa bits (|x| < 2^-126 to 0)
+__device__ __forceinline__ float cut(float x) { return x; }
+__device__ __forceinline__ float cut(double x) {
+    const int hi = __double2hiint(x);
+    const unsigned int a = max(hi & 0x7fffffff, 0x38000000) - 0x38000000;
+    return __uint_as_float((a << 3) | (hi & 0x80000000u));
+}
+
+// PPW: particles per warp, 32 (one lane each) or 8 (four lanes share a
+// particle: lane t takes entry t of every group).  Returns the pair force on the
+// lane's particle (PPW 8: on each of its four lanes); pe, vir, vxz: sums over the
+// pairs this lane evaluated.
+template <class T, bool ENERGY, bool MULTI, bool FAST, bool DPD, bool LE, int PPW>
+__device__ __forceinline__ void queue_loop(const DevSys<T>& s, const V4<T>* __restrict__ P,
+                                           PairQueue<T, DPD, PPW>& Q, int ibase, int i, int n, const RepGeom<T>& g,
+                                           const V4<T>& xi, const PairRec<T>* pr1, T rcmax2, const LeCtx<T>& le,
+                                           long long step, T& fx, T& fy, T& fz, T& pe, T& vir, T& vxz) {
+    constexpr int TPP = 32 / PPW;         // lanes per particle
+    constexpr int QG = PairQueue<T, DPD, PPW>::QG, QR = PairQueue<T, DPD, PPW>::QR;
+    constexpr int C = TPP == 1 ? 4 : 1;   // entries of a group per lane
+    static_assert(TPP == 1 || TPP == 4, "one or four lanes per particle");
+    const int lane = threadIdx.x & 31, t0 = TPP == 1 ? 0 : lane & 3;
+    int* __restrict__ col = Q.col + (TPP == 1 ? lane : lane >> 2);
+    const float L0 = (float)g.L[0], L1 = (float)g.L[1], L2 = (float)g.L[2];
+    const float x = cut(xi.x), y = cut(xi.y), z = cut(xi.z);
+    float rc2;
+    if constexpr (sizeof(T) == 4) {
+        rc2 = rcmax2;
+    } else {
+        // every component is off by at most 2^-20 of a coordinate on either
+        // side (and by its image shift's rounding)
+        const float r2 = (float)rcmax2, r = sqrtf(r2), e = 3e-6f * (fmaxf(L0, fmaxf(L1, L2)) + 2.f * (float)s.skin);
+        rc2 = (r2 + 3.47f * r * e + 3.f * e * e) * 1.00001f;
+    }
+    const float led = (float)le.d, linv = (float)le.inv_Lx;
+    const int ng = (n + 3) >> 2;
+    const int ngw = __reduce_max_sync(0xffffffffu, ng);
+    const size_t stride = (size_t)s.stride;
+    const int pad = s.nbr_pad;
+    const int4* __restrict__ nb4 = reinterpret_cast<const int4*>(s.nbr) + i;
+    const int* __restrict__ nb1 = s.nbr + 4 * (size_t)i + t0;
+    for (int g0 = 0; g0 < ngw; g0 += QG) {
+        int cnt = 0;  // entries in the particle's column
+        const int g1 = min(g0 + QG, ngw);
+        // ---- the entries inside the (widened) cutoff
+#pragma unroll 2
+        for (int q = g0; q < g1; ++q) {
+            int e[C];
+            if constexpr (C == 4) {
+                const int4 a = q < ng ? __ldg(nb4 + q * stride) : make_int4(pad, pad, pad, pad);
+                e[0] = a.x;
+                e[1 % C] = a.y;
+                e[2 % C] = a.z;
+                e[3 % C] = a.w;
+            } else {
+                e[0] = q < ng ? __ldg(nb1 + 4 * (size_t)q * stride) : pad;
+            }
+            V4<T> xj[C];
+#pragma unroll
+            for (int t = 0; t < C; ++t) xj[t] = ld4<T>(P + nbr_slot(e[t]));
+#pragma unroll
+            for (int t = 0; t < C; ++t) {
+                const int code = nbr_code(e[t]);
+                const float xq = cut(xj[t].x), yq = cut(xj[t].y), zq = cut(xj[t].z);
+                float dx = x - xq, dy = y - yq, dz = z - zq;
+                if (code != 0) {
+                    dx = shifted_diff(x, x - L0, xq, L0, code & 3);
+                    dy = shifted_diff(y, y - L1, yq, L1, (code >> 2) & 3);
+                    dz = shifted_diff(z, z - L2, zq, L2, code >> 4);
+                    if (LE && (code & 3) == 3) dx = le_dx(x, xq, (code >> 4) == 1 ? 1 : -1, led, L0, linv);
+                }
+                const bool in = dx * dx + dy * dy + dz * dz < rc2;
+                if constexpr (TPP == 1) {
+                    if (in) {
+                        col[cnt * PPW] = e[t];
+                        ++cnt;
+                    }
+                } else {
+                    const unsigned int m = (__ballot_sync(0xffffffffu, in) >> (lane & 28)) & 15u;
+                    if (in) col[(cnt + __popc(m & ((1u << t0) - 1u))) * PPW] = e[t];
+                    cnt += __popc(m);
+                }
+            }
+        }
+        // where each particle's terms start in the warp's queue
+        int off = t0 == 0 ? cnt : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, off, o);
+            if (lane >= o) off += u;
+        }
+        const int total = __shfl_sync(0xffffffffu, off, 31);
+        if (t0 == 0) off -= cnt;
+        const int from = TPP == 1 ? off : __shfl_sync(0xffffffffu, off, lane & 28), to = from + cnt;
+        for (int r0 = 0; r0 < total; r0 += QR) {
+            const int nr = min(QR, total - r0);
+            __syncwarp();
+            for (int b = 0; b < nr; b += 32) {
+                const int q = min(b + lane, nr - 1) + r0;
+                // the particle of entry q: the last lane whose terms start at or before q
+                int own = 0;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+                    if (__shfl_sync(0xffffffffu, off, own + o) <= q) own += o;
+                const int k = q - __shfl_sync(0xffffffffu, off, own);
+                if (b + lane < nr) {
+                    const int p = TPP == 1 ? own : own >> 2;
+                    const int e = Q.col[k * PPW + p];
+                    const int ii = ibase + p, j = nbr_slot(e), code = nbr_code(e);
+                    const V4<T> a = ld4<T>(P + ii), xj = ld4<T>(P + j);
+                    int nz = 0;
+                    T dx, dy, dz;
+                    if (code == 0) {
+                        dx = a.x - xj.x;
+                        dy = a.y - xj.y;
+                        dz = a.z - xj.z;
+                    } else {
+                        if (LE && (code & 3) == 3) {
+                            nz = (code >> 4) == 1 ? 1 : -1;
+                            dx = le_dx(a.x, xj.x, nz, le.d, g.L[0], le.inv_Lx);
+                        } else {
+                            dx = shifted_diff(a.x, a.x - g.L[0], xj.x, g.L[0], code & 3);
+                        }
+                        dy = shifted_diff(a.y, a.y - g.L[1], xj.y, g.L[1], (code >> 2) & 3);
+                        dz = shifted_diff(a.z, a.z - g.L[2], xj.z, g.L[2], code >> 4);
+                    }
+                    const T r2 = dx * dx + dy * dy + dz * dz;
+                    Q.fr[b + lane] = pair_scalar<T, ENERGY, MULTI, FAST>(s, MULTI ? bits_as_int(a.w) : 0, pr1, dx, dz, r2,
+                                                                         bits_as_int(xj.w), pe, vir, vxz);
+                    Q.dx[b + lane] = dx;
+                    Q.dy[b + lane] = dy;
+                    Q.dz[b + lane] = dz;
+                    if (DPD) {
+                        T th = T(0);
+                        if (less_nonneg(r2, s.ip->dpd_rc2)) {
+                            DpdCtx<T> dc;
+                            dc.vi = ld4<T>(s.vsnap + ii);
+                            dc.seed = g.seed;
+                            dc.step = step;
+                            dc.le_vs = le.vs;
+                            th = dpd_value<T>(s.ip, dc, dx, dy, dz, r2, ld4<T>(s.vsnap + j), nz);
+                        }
+                        Q.th[b + lane] = th;
+                    }
+                }
+            }
+            __syncwarp();
+            const int k0 = max(from, r0) - r0, k1 = min(to, r0 + nr) - r0;
+            if constexpr (TPP == 1) {
+                for (int k = k0; k < k1; ++k) {
+                    const T fr = Q.fr[k], dx = Q.dx[k], dy = Q.dy[k], dz = Q.dz[k];
+                    fx = fma_rn(fr, dx, fx);
+                    fy = fma_rn(fr, dy, fy);
+                    fz = fma_rn(fr, dz, fz);
+                    if (DPD) {
+                        const T th = Q.th[k];
+                        fx = fma_rn(th, dx, fx);
+                        fy = fma_rn(th, dy, fy);
+                        fz = fma_rn(th, dz, fz);
+                    }
+                }
+            } else {
+                // one component per lane
+                const T* d = t0 == 0 ? Q.dx : t0 == 1 ? Q.dy : Q.dz;
+                for (int k = k0; k < k1; ++k) {
+                    const T dd = d[k];
+                    fx = fma_rn(Q.fr[k], dd, fx);
+                    if (DPD) fx = fma_rn(Q.th[k], dd, fx);
+                }
+            }
+        }
+        __syncwarp();
+    }
+    if constexpr (TPP == 4) {
+        const T f = fx;
+        fx = __shfl_sync(0xffffffffu, f, lane & 28);
+        fy = __shfl_sync(0xffffffffu, f, (lane & 28) + 1);
+        fz = __shfl_sync(0xffffffffu, f, (lane & 28) + 2);
     }
 }
 
@@ -262,8 +455,9 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// SH: launch shape (STEP_SHAPES) of the plain FP32 list path.
-template <class T, int MODE, bool ENERGY, bool FAST, bool DPD, bool LE, int SH = 0>
+// SH: launch shape (STEP_SHAPES) of the plain FP32 list path.  PPW: particles
+// per warp of the queue path (32, or 8 with four lanes per particle).
+template <class T, int MODE, bool ENERGY, bool FAST, bool DPD, bool LE, int SH = 0, int PPW = 32>
 __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
                                   sizeof(T) == 4 ? (DPD ? ESPP_STEP_MINB32_DPD
                                                         : (SH == 0 ? ESPP_STEP_MINB32 : STEP_SHAPES[SH].minb))
@@ -273,9 +467,14 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
     // is written for one
     constexpr int TPB = STEP_SHAPES[SH].tpb;
     static_assert(TPB == 1 || !ENERGY, "energy reductions take one tile per block");
-    const int lt = TPB > 1 ? (int)threadIdx.x % TILE : (int)threadIdx.x;  // index inside the tile
+    static_assert(PPW == 32 || (TPB == 1 && !ENERGY), "four lanes per particle: single tiles, no reductions");
+    constexpr bool QUEUE = sizeof(T) == 8 || DPD;
+    constexpr int TPP = 32 / PPW;  // lanes per particle, blocks per tile
+    // index inside the tile
+    const int lt = TPP > 1 ? (int)(blockIdx.x % TPP) * (TILE / TPP) + (int)threadIdx.x / TPP
+                 : TPB > 1 ? (int)threadIdx.x % TILE : (int)threadIdx.x;
     Ctrl* c = s.ctrl;
-    const int t0 = blockIdx.x * TPB + (TPB > 1 ? (int)threadIdx.x / TILE : 0);
+    const int t0 = TPP > 1 ? blockIdx.x / TPP : blockIdx.x * TPB + (TPB > 1 ? (int)threadIdx.x / TILE : 0);
     // the first tile's record is requested together with the abort flag
     Tile tl0 = {0, 0, 0, 0};
     if (t0 < s.ntiles) tl0 = ld_tile_early(s.tiles + t0);
@@ -285,8 +484,9 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
     V4<T>* __restrict__ Pn = s.pos[cur ^ 1];
     const IntParams<T>* __restrict__ ip = s.ip;
     __shared__ double red[NPART][TILE / 32];
+    __shared__ __align__(16) unsigned char queue_mem[QUEUE ? sizeof(PairQueue<T, DPD, PPW>) * (TILE / 32) : 16];
 
-    for (int t = t0; t < s.ntiles; t += gridDim.x * TPB) {
+    for (int t = t0; t < s.ntiles; t += TPP > 1 ? s.ntiles : gridDim.x * TPB) {
         const Tile tl = t == t0 ? tl0 : s.tiles[t];
         const bool active = lt < tl.count;
         const RepGeom<T>& g = s.reps[tl.rep];
@@ -320,22 +520,43 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
         } else {
             le.d = le.inv_Lx = le.vs = le.shear = T(0);
         }
-        if (active) {
-            const int i = tl.start + lt;
-            const T L0 = g.L[0], L1 = g.L[1], L2 = g.L[2];
+        // a warp's queue takes all of its lanes: those without a particle
+        // stand at the tile's first one with an empty list
+        const int i = tl.start + (active ? lt : 0);
+        const T L0 = g.L[0], L1 = g.L[1], L2 = g.L[2];
+        T fx = 0, fy = 0, fz = 0, pe = 0, pb = 0, vir = 0, vxz = 0;
+        double blen = 0.0, bcnt = 0.0;
+        if constexpr (QUEUE) {
+            if (!s.mlp_on && (FAST || !s.cells_mode)) {
+                const V4<T> xi = ld4<T>(P + i);
+                const int n = active ? s.nbr_cnt[i] : 0;
+                PairQueue<T, DPD, PPW>& q = reinterpret_cast<PairQueue<T, DPD, PPW>*>(queue_mem)[threadIdx.x >> 5];
+                const int ibase = tl.start + lt / PPW * PPW;
+                T rcmax2 = s.rc_max2;
+                if (DPD) rcmax2 = max(rcmax2, s.ip->dpd_rc2);
+                if (FAST || s.ntypes == 1) {
+                    const PairRec<T> pr = s.pair[0];
+                    queue_loop<T, ENERGY, false, FAST, DPD, LE, PPW>(s, P, q, ibase, i, n, g, xi, &pr, rcmax2, le, step,
+                                                                    fx, fy, fz, pe, vir, vxz);
+                } else {
+                    queue_loop<T, ENERGY, true, false, DPD, LE, PPW>(s, P, q, ibase, i, n, g, xi, nullptr, rcmax2, le,
+                                                                    step, fx, fy, fz, pe, vir, vxz);
+                }
+            }
+        }
+        if (active && (TPP == 1 || threadIdx.x % TPP == 0)) {
             const T H0 = g.halfL[0], H1 = g.halfL[1], H2 = g.halfL[2];
             // independent loads first: own position, list count, bond slots,
             // velocity and build position, then the bond partners' positions
             const V4<T> xi = ld4<T>(P + i);
             const int ti = bits_as_int(xi.w);
-            T fx = 0, fy = 0, fz = 0, pe = 0, pb = 0, vir = 0, vxz = 0;
             const int n = s.nbr_cnt[i];
             const bool bonded = s.bond.kind != 0;
             const int2 b = bonded ? s.bond_slot[i] : make_int2(-1, -1);
             // loads the pair loop does not need, issued before it (latency
             // hidden behind the loop) or after it (fewer registers held)
             constexpr bool LATE_BOND = (ESPP_STEP_LATE & 1) != 0;
-            constexpr bool LATE_VEL = (ESPP_STEP_LATE & 2) != 0 && !DPD;
+            constexpr bool LATE_VEL = (ESPP_STEP_LATE & 2) != 0;
             V4<T> v, xbi, xp0, xp1;
             if (!LATE_VEL) {
                 v = s.vel[i];
@@ -344,13 +565,6 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
             if (!LATE_BOND) {
                 xp0 = b.x >= 0 ? ld4<T>(P + b.x) : xi;
                 xp1 = b.y >= 0 ? ld4<T>(P + b.y) : xi;
-            }
-            DpdCtx<T> dc;
-            if (DPD) {
-                dc.vi = v;
-                dc.seed = g.seed;
-                dc.step = step;
-                dc.le_vs = le.vs;
             }
             if (s.mlp_on) {
                 // pair forces of the learned potential, computed by k_mlp
@@ -374,7 +588,14 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
                         vir = (T)s.mlp_w[i];
                     }
                 }
-                if (DPD) dpd_loop<T, LE>(s, P, i, n, xi, dc, le, L0, L1, L2, fx, fy, fz);
+                if (DPD) {
+                    DpdCtx<T> dc;
+                    dc.vi = s.vel[i];
+                    dc.seed = g.seed;
+                    dc.step = step;
+                    dc.le_vs = le.vs;
+                    dpd_loop<T, LE>(s, P, i, n, xi, dc, le, L0, L1, L2, fx, fy, fz);
+                }
             } else if (!FAST && s.cells_mode) {
                 // list-free mode: pair forces (with the DPD pair term) from
                 // the cell-stencil kernel
@@ -388,25 +609,27 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
                     vir = w.x;
                     vxz = w.y;
                 }
-            } else if (FAST) {
-                PairRec<T> pr;
-                pr.rc2 = s.pair[0].rc2;
-                pr.sig2 = s.pair[0].sig2;
-                pr.eps24 = s.pair[0].eps24;
-                if (ENERGY) {
-                    pr.eps4 = s.pair[0].eps4;
-                    pr.shift = s.pair[0].shift;
+            } else if constexpr (!QUEUE) {
+                if (FAST) {
+                    PairRec<T> pr;
+                    pr.rc2 = s.pair[0].rc2;
+                    pr.sig2 = s.pair[0].sig2;
+                    pr.eps24 = s.pair[0].eps24;
+                    if (ENERGY) {
+                        pr.eps4 = s.pair[0].eps4;
+                        pr.shift = s.pair[0].shift;
+                    }
+                    pair_loop<T, ENERGY, false, true, LE, STEP_SHAPES[SH].groups>(s, P, i, n, xi, ti, &pr, L0, L1, L2, fx,
+                                                                                  fy, fz, pe, vir, vxz, &le);
+                } else if (s.ntypes == 1) {
+                    const PairRec<T> pr = s.pair[0];
+                    if (pr.kind != 0)
+                        pair_loop<T, ENERGY, false, false, LE>(s, P, i, n, xi, ti, &pr, L0, L1, L2, fx, fy, fz, pe, vir,
+                                                               vxz, &le);
+                } else {
+                    pair_loop<T, ENERGY, true, false, LE>(s, P, i, n, xi, ti, nullptr, L0, L1, L2, fx, fy, fz, pe, vir,
+                                                          vxz, &le);
                 }
-                pair_loop<T, ENERGY, false, true, DPD, LE, STEP_SHAPES[SH].groups>(s, P, i, n, xi, ti, &pr, L0, L1, L2,
-                                                                                   fx, fy, fz, pe, vir, vxz, &le, &dc);
-            } else if (s.ntypes == 1) {
-                const PairRec<T> pr = s.pair[0];
-                if (pr.kind != 0 || DPD)
-                    pair_loop<T, ENERGY, false, false, DPD, LE>(s, P, i, n, xi, ti, &pr, L0, L1, L2, fx, fy, fz, pe,
-                                                            vir, vxz, &le, &dc);
-            } else {
-                pair_loop<T, ENERGY, true, false, DPD, LE>(s, P, i, n, xi, ti, nullptr, L0, L1, L2, fx, fy, fz, pe,
-                                                       vir, vxz, &le, &dc);
             }
             if (LATE_VEL) {
                 v = s.vel[i];
@@ -417,7 +640,6 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
                 xp1 = b.y >= 0 ? ld4<T>(P + b.y) : xi;
             }
             // bonds (paper "Functionality": bonded interactions; FENE or tabulated)
-            double blen = 0.0, bcnt = 0.0;
             if (bonded) {
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
@@ -437,7 +659,7 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
                     T fr, ub = T(0);
                     if (s.bond.kind == ESPP_FENE) {
                         T one_m = T(1) - r2 * s.bond.inv_R02;
-                        if (!(one_m > T(0))) {
+                        if (!positive(one_m)) {
                             atomicOr(&c->err, ERRBIT_BOND);
                             c->abort = 1;
                             __threadfence();
@@ -467,14 +689,6 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
                         bcnt += 1.0;
                     }
                 }
-            }
-            if (ENERGY) {
-                acc[P_PE_PAIR] = 0.5 * (double)pe;
-                acc[P_PE_BOND] = 0.5 * (double)pb;
-                acc[P_VIRIAL] = 0.5 * (double)vir;
-                acc[P_BOND_LEN] = 0.5 * blen;
-                acc[P_BOND_CNT] = 0.5 * bcnt;
-                acc[P_VIR_XZ] = 0.5 * (double)vxz;
             }
             if (MODE == MODE_FORCES) {
                 if (f_out) {
@@ -524,7 +738,7 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
                         T x = drift(xi.x, v.x, dt), y = drift(xi.y, v.y, dt), z = drift(xi.z, v.z, dt);
                         // no wrap here: positions stay in the image frame of the
                         // last list build until the next build wraps them
-                        if (!(fabs(x) < T(1e30) && fabs(y) < T(1e30) && fabs(z) < T(1e30))) {
+                        if (!(abs_less(x, T(1e30)) && abs_less(y, T(1e30)) && abs_less(z, T(1e30)))) {
                             atomicOr(&c->err, ERRBIT_NONFINITE);
                             c->abort = 1;
                             __threadfence();
@@ -539,7 +753,7 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
                             }
                         } else {
                             const T ex = x - xbi.x, ey = y - xbi.y, ez = z - xbi.z;
-                            if (ex * ex + ey * ey + ez * ez > skin_thr2) {
+                            if (less_nonneg(skin_thr2, ex * ex + ey * ey + ez * ez)) {
                                 s.req[tl.rep] = 1;
                                 c->any_req = 1;
                                 __threadfence();
@@ -552,6 +766,13 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
             }
         }
         if (ENERGY) {
+            // the queue's lanes hold the pairs they evaluated, whosever they are
+            acc[P_PE_PAIR] = 0.5 * (double)pe;
+            acc[P_PE_BOND] = 0.5 * (double)pb;
+            acc[P_VIRIAL] = 0.5 * (double)vir;
+            acc[P_BOND_LEN] = 0.5 * blen;
+            acc[P_BOND_CNT] = 0.5 * bcnt;
+            acc[P_VIR_XZ] = 0.5 * (double)vxz;
             const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
             for (int k = 0; k < NPART; ++k) {
@@ -622,7 +843,7 @@ __global__ void __launch_bounds__(TILE) k_prologue(DevSys<T> s, int cur) {
         v.z = half_kick(v.z, f.z, hdt, inv_m);
         const T dt = ip->dt;
         T x = drift(xi.x, v.x, dt), y = drift(xi.y, v.y, dt), z = drift(xi.z, v.z, dt);
-        if (!(fabs(x) < T(1e30) && fabs(y) < T(1e30) && fabs(z) < T(1e30))) {
+        if (!(abs_less(x, T(1e30)) && abs_less(y, T(1e30)) && abs_less(z, T(1e30)))) {
             atomicOr(&c->err, ERRBIT_NONFINITE);
             c->abort = 1;
             x = xi.x; y = xi.y; z = xi.z;
@@ -634,7 +855,7 @@ __global__ void __launch_bounds__(TILE) k_prologue(DevSys<T> s, int cur) {
         } else {
             const V4<T> b = s.xb[i];
             const T ex = x - b.x, ey = y - b.y, ez = z - b.z;
-            if (ex * ex + ey * ey + ez * ez > skin_thr2) {
+            if (less_nonneg(skin_thr2, ex * ex + ey * ey + ez * ez)) {
                 s.req[tl.rep] = 1;
                 c->any_req = 1;
             }
@@ -649,6 +870,18 @@ __global__ void k_set_cond(DevSys<T> s, unsigned long long h) {
     const unsigned int want = *(volatile unsigned int*)&s.ctrl->any_req;
     const unsigned int ab = *(volatile unsigned int*)&s.ctrl->abort;
     cudaGraphSetConditional(h, (want && !ab) ? 1u : 0u);
+}
+
+// Four lanes per particle on the queue path while one lane per particle leaves
+// SMs idle, and on long lists, whose eight-particle queues are full anyway.
+// Step kernel (event-timed), one lane / four: KG melt FP64 1,000 25.4 / 16.6 us,
+// 5,000 27.8 / 20.9, 10,000 28.8 / 27.0, 20,000 29.6 / 40, 40,000 39 / 58; LJ
+// fluid FP64 (76 entries) 27,436 194 / 137, 256,000 1186 / 822; DPD fluid FP32
+// 24,000 47 / 27, 98,304 56 / 62.
+template <class T>
+static bool queue_spread(const DevSys<T>& s) {
+    if (sizeof(T) == 8) return s.N < 12288 || s.cap >= 64;
+    return s.N < 49152;
 }
 
 template <class T>
@@ -667,6 +900,18 @@ int Launch<T>::step(const DevSys<T>& s, int mode, bool energy, int cur, double* 
     // the plain FP32 list path of a step takes the tuned launch shape
     const int sh = (sizeof(T) == 4 && s.lj_fast && !s.le_on && !s.cells_mode && !s.mlp_on &&
                     (mode == MODE_STEP || mode == MODE_FINAL) && !dpd) ? s.step_shape : 0;
+    // queue path of a small handle: four lanes per particle (see the rule above)
+    const bool spread = (sizeof(T) == 8 || dpd) && !s.mlp_on && !s.cells_mode && queue_spread(s);
+#define ESPP_STEP_Q(M, E, F, D, LE)                                                                        \
+    do {                                                                                                   \
+        if constexpr ((sizeof(T) == 8 || (D)) && !(E)) {                                                   \
+            if (spread) {                                                                                  \
+                k_step<T, M, E, F, D, LE, 0, 8><<<4 * s.ntiles, TILE, 0, st>>>(s, cur, f_out, next_cond);  \
+                break;                                                                                     \
+            }                                                                                              \
+        }                                                                                                  \
+        k_step<T, M, E, F, D, LE><<<gr, TILE, 0, st>>>(s, cur, f_out, next_cond);                          \
+    } while (0)
 #define ESPP_STEP_SHAPED(M, E, D, LE, K)                                                                   \
     k_step<T, M, E, true, D, LE, K>                                                                        \
         <<<(gr + STEP_SHAPES[K].tpb - 1) / STEP_SHAPES[K].tpb, TILE * STEP_SHAPES[K].tpb, 0, st>>>(s, cur, f_out, next_cond)
@@ -685,12 +930,12 @@ int Launch<T>::step(const DevSys<T>& s, int mode, bool energy, int cur, double* 
             }                                                                                              \
             if (sh != 0) break;                                                                            \
         }                                                                                                  \
-        k_step<T, M, E, true, D, LE><<<gr, TILE, 0, st>>>(s, cur, f_out, next_cond);                       \
+        ESPP_STEP_Q(M, E, true, D, LE);                                                                    \
     } while (0)
 #define ESPP_STEP_LE(M, E, D, LE)                                                                \
     do {                                                                                         \
         if (s.lj_fast) ESPP_STEP_SH(M, E, D, LE);                                                \
-        else k_step<T, M, E, false, D, LE><<<gr, TILE, 0, st>>>(s, cur, f_out, next_cond);         \
+        else ESPP_STEP_Q(M, E, false, D, LE);                                                    \
     } while (0)
 #define ESPP_STEP(M, E, D)                            \
     do {                                              \
@@ -712,6 +957,7 @@ int Launch<T>::step(const DevSys<T>& s, int mode, bool energy, int cur, double* 
             break;
     }
 #undef ESPP_STEP
+#undef ESPP_STEP_Q
 #undef ESPP_STEP_LE
 #undef ESPP_STEP_SH
 #undef ESPP_STEP_SHAPED

@@ -18,11 +18,10 @@
 // half issue (55%) and half the L1 data pipe (68%: each candidate is a 16-byte
 // gather of its own).
 //
-// FP64 handles test the candidates in FP32 first, on float copies of the
-// entries and against a radius widened by the error of those coordinates, and
-// evaluate the exact FP64 test on what is left when a column is written out:
-// the same list, with the FP64 unit busy for about as many pairs as the list
-// holds instead of all candidates.
+// FP64 handles test the candidates in FP32, on float copies of the entries; a
+// candidate nearer to the list radius than those coordinates' error is marked
+// and gets the exact FP64 test when its column is written out: the same list,
+// with the FP64 unit idle but for a few pairs in a hundred thousand.
 #include "kernels.cuh"
 
 namespace espp {
@@ -54,7 +53,7 @@ template <class T, int W, bool EXCL, bool LE, int TS>
 struct VerletSearch {
     const DevSys<T>& s;
     const RepGeom<T>& g;
-    const float4* __restrict__ EF;  // entries in FP32 (x, y, z, slot bits in FP32 handles)
+    const float4* __restrict__ EF;  // entries in FP32 (x, y, z, slot bits)
     int* col;
     int idx;        // the particle's own entry
     int i;          // its storage slot
@@ -66,6 +65,8 @@ struct VerletSearch {
     int cnt = 0;    // entries waiting in the column
     int done = 0;   // whole groups written
     float rl2f;     // list radius^2 of the FP32 test
+    float rl2in;    // FP64 handles: below it the FP32 test is certain
+    const V4<T>* __restrict__ P;
     T le_d = T(0), inv_L0 = T(0);
     int4* __restrict__ out4;
 
@@ -104,9 +105,11 @@ struct VerletSearch {
                 const float dy = SHIFT ? yo - (x[k].y - yL) : yo - x[k].y;
                 const float dz = SHIFT ? zo - (x[k].z - zL) : zo - x[k].z;
                 const int j = __float_as_int(x[k].w);
-                bool hit = dx * dx + dy * dy + dz * dz < rl2f && q != idx && (q < e || (TS == 1 && k == 0));
-                if (EXCL && EXACT) hit = hit && j != ex.x && j != ex.y;
-                const int val = (EXACT ? j : q) | tag;
+                const float r2 = dx * dx + dy * dy + dz * dz;
+                bool hit = r2 < rl2f && q != idx && (q < e || (TS == 1 && k == 0));
+                if (EXCL) hit = hit && j != ex.x && j != ex.y;
+                int val = j | tag;
+                if (!EXACT && !(r2 < rl2in)) val |= (int)0x80000000;  // too near the list radius to tell
                 if constexpr (TS == 1) {
                     if (hit) {
                         col[cnt * CS] = val;
@@ -122,12 +125,11 @@ struct VerletSearch {
         }
     }
 
-    // FP64 handles: the exact test of the waiting entries (entry index and
-    // image code), which become list entries (slot and code) in place
-    __device__ __forceinline__ bool exact_hit(int v, int& entry) {
-        const int p = v & NBR_INDEX_MASK, code = v >> NBR_INDEX_BITS;
-        const V4<T> xj = ld4<T>(s.cell_ent + p);
-        const int j = bits_as_int(xj.w);
+    // FP64 handles: the exact test of a waiting entry too near the list radius
+    // for the FP32 one
+    __device__ __forceinline__ bool exact_hit(int v) const {
+        const int code = (v & 0x7fffffff) >> NBR_INDEX_BITS;
+        const V4<T> xj = ld4<T>(P + nbr_slot(v));
         T dx;
         if (LE && (code & 3) == 3) {
             const T nd = (code >> 4) == 1 ? le_d : -le_d;
@@ -138,41 +140,34 @@ struct VerletSearch {
         }
         const T dy = shifted_diff(xi.y, xi.y - g.L[1], xj.y, g.L[1], (code >> 2) & 3);
         const T dz = shifted_diff(xi.z, xi.z - g.L[2], xj.z, g.L[2], code >> 4);
-        bool hit = dx * dx + dy * dy + dz * dz < s.rlist2;
-        if (EXCL) hit = hit && j != ex.x && j != ex.y;
-        entry = j | (v & ~NBR_INDEX_MASK);
-        return hit;
+        return dx * dx + dy * dy + dz * dz < s.rlist2;
     }
 
-    int tested = 0;  // leading entries of the column that passed the exact test
-
+    // the waiting entries that belong to the list, in place
     __device__ __forceinline__ void settle() {
         if constexpr (!EXACT) {
             if constexpr (TS == 1) {
-                int w = tested;
-                for (int k = tested; k < cnt; ++k) {
-                    int en;
-                    if (exact_hit(col[k * CS], en)) {
-                        col[w * CS] = en;
-                        ++w;
-                    }
+                int w = 0;
+                for (int k = 0; k < cnt; ++k) {
+                    const int v = col[k * CS];
+                    if (v < 0 && !exact_hit(v)) continue;
+                    col[w * CS] = v & 0x7fffffff;
+                    ++w;
                 }
                 cnt = w;
             } else {
                 __syncwarp(tmask);
-                int w = tested;
-                for (int k = tested; k < cnt; k += TS) {
-                    int en = 0;
-                    bool hit = false;
-                    if (k + sub < cnt) hit = exact_hit(col[k + sub], en);
-                    const unsigned int m = __ballot_sync(tmask, hit) & tmask;
-                    if (hit) col[w + __popc(m & ((1u << (threadIdx.x & 31)) - 1u))] = en;
+                int w = 0;
+                for (int k = 0; k < cnt; k += TS) {
+                    const int v = k + sub < cnt ? col[k + sub] : 0;
+                    const bool keep = k + sub < cnt && (v >= 0 || exact_hit(v));
+                    const unsigned int m = __ballot_sync(tmask, keep) & tmask;
+                    if (keep) col[w + __popc(m & ((1u << (threadIdx.x & 31)) - 1u))] = v & 0x7fffffff;
                     w += __popc(m);
                     __syncwarp(tmask);
                 }
                 cnt = w;
             }
-            tested = cnt;
         }
     }
 
@@ -202,7 +197,6 @@ struct VerletSearch {
             __syncwarp(tmask);
             cnt = r;
         }
-        tested = cnt;
         done += ng;
     }
 
@@ -355,7 +349,9 @@ struct VerletSearch {
             // again where a sheared image is taken
             const float Lm = (float)fmax((double)g.L[0], fmax((double)g.L[1], (double)g.L[2]));
             const float r2 = (float)s.rlist2, r = sqrtf(r2), e = 6e-7f * (Lm + r);
-            rl2f = (r2 + 2.f * 1.7320509f * r * e + 3.f * e * e) * 1.000001f;
+            const float m = 2.f * 1.7320509f * r * e + 3.f * e * e;
+            rl2f = (r2 + m) * 1.000001f;
+            rl2in = (r2 - m) * 0.999999f;
         }
         if (W > 1) {
             cpl0 = (float)g.cells_per_len[0];
@@ -393,7 +389,7 @@ struct VerletSearch {
 // One thread per particle, threads in entry (cell) order: a warp walks a run of
 // cells along x, whose stencils share their rows.
 template <class T, int W, bool EXCL, bool LE>
-__global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? 8 : 6) k_verlet(DevSys<T> s) {
+__global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? 8 : 6) k_verlet(DevSys<T> s, int cur) {
     __shared__ int buf[TILE / 32][VB * 32];
     // the first tile's record is requested together with the abort flag
     Tile tl0 = {0, 0, 0, 0};
@@ -404,6 +400,7 @@ __global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? 8 : 6) k_verlet(DevSys<
         if (!s.now[tl.rep]) continue;  // uniform over the block
         VerletSearch<T, W, EXCL, LE, 1> v(s, s.reps[tl.rep]);
         v.EF = entries_f(s);
+        v.P = s.pos[cur];
         v.col = buf[threadIdx.x >> 5] + (threadIdx.x & 31);
         v.sub = 0;
         v.tmask = 0;
@@ -423,7 +420,7 @@ __global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? 8 : 6) k_verlet(DevSys<
 // VTEAM lanes per particle (TILE / VTEAM particles per block), for systems that
 // do not fill the chip with one thread per particle.
 template <class T, int W, bool EXCL, bool LE>
-__global__ void __launch_bounds__(TILE, 6) k_verlet_team(DevSys<T> s) {
+__global__ void __launch_bounds__(TILE, 6) k_verlet_team(DevSys<T> s, int cur) {
     __shared__ __align__(16) int buf[TILE / VTEAM][VTB];
     if (s.ctrl->abort) return;
     const int t = blockIdx.x / VTEAM;
@@ -435,6 +432,7 @@ __global__ void __launch_bounds__(TILE, 6) k_verlet_team(DevSys<T> s) {
     if (q >= tl.count) return;   // whole teams
     VerletSearch<T, W, EXCL, LE, VTEAM> v(s, s.reps[tl.rep]);
     v.EF = entries_f(s);
+    v.P = s.pos[cur];
     v.col = buf[team];
     v.sub = lane % VTEAM;
     v.tmask = ((1u << VTEAM) - 1u) << (lane / VTEAM * VTEAM);
@@ -445,16 +443,16 @@ __global__ void __launch_bounds__(TILE, 6) k_verlet_team(DevSys<T> s) {
 }
 
 template <class T>
-void Launch<T>::verlet(const DevSys<T>& s, cudaStream_t st) {
+void Launch<T>::verlet(const DevSys<T>& s, int cur, cudaStream_t st) {
     const bool team = s.N < verlet_team_below<T>();
 #define ESPP_VERLET(W, E)                                                                                  \
     do {                                                                                                   \
         if (team) {                                                                                        \
-            if (s.le_on) k_verlet_team<T, W, E, true><<<s.ntiles * VTEAM, TILE, 0, st>>>(s);               \
-            else k_verlet_team<T, W, E, false><<<s.ntiles * VTEAM, TILE, 0, st>>>(s);                      \
+            if (s.le_on) k_verlet_team<T, W, E, true><<<s.ntiles * VTEAM, TILE, 0, st>>>(s, cur);               \
+            else k_verlet_team<T, W, E, false><<<s.ntiles * VTEAM, TILE, 0, st>>>(s, cur);                      \
         } else {                                                                                           \
-            if (s.le_on) k_verlet<T, W, E, true><<<s.ntiles, TILE, 0, st>>>(s);                            \
-            else k_verlet<T, W, E, false><<<s.ntiles, TILE, 0, st>>>(s);                                   \
+            if (s.le_on) k_verlet<T, W, E, true><<<s.ntiles, TILE, 0, st>>>(s, cur);                            \
+            else k_verlet<T, W, E, false><<<s.ntiles, TILE, 0, st>>>(s, cur);                                   \
         }                                                                                                  \
     } while (0)
 #define ESPP_VERLET_W(E)                    \
@@ -470,10 +468,10 @@ void Launch<T>::verlet(const DevSys<T>& s, cudaStream_t st) {
 }
 
 #if !defined(ESPP_STEP_PRECISION) || ESPP_STEP_PRECISION == 32
-template void Launch<float>::verlet(const DevSys<float>&, cudaStream_t);
+template void Launch<float>::verlet(const DevSys<float>&, int, cudaStream_t);
 #endif
 #if !defined(ESPP_STEP_PRECISION) || ESPP_STEP_PRECISION == 64
-template void Launch<double>::verlet(const DevSys<double>&, cudaStream_t);
+template void Launch<double>::verlet(const DevSys<double>&, int, cudaStream_t);
 #endif
 
 }  // namespace espp

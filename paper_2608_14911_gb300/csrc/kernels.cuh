@@ -85,7 +85,7 @@ template <class T> struct DevSys {
     // compact entries (position, storage slot in the w lane): those of cell h
     // are cell_ent[cell_beg[h] .. cell_beg[h + 1]), ascending slot
     V4<T>* cell_ent;
-    float4* cell_ent32;     // FP64 handles: the entries' coordinates in FP32 (list search)
+    float4* cell_ent32;     // FP64 handles: the entries in FP32 (list search)
     int* cell_beg;          // ncells + 1; cell_beg[ncells] = N
     int* rank_start;        // first new slot of each cell in Hilbert-rank order (resort only)
     int cell_w;             // cell subdivision: cells of edge >= (rc + skin) / cell_w (1, 2 or 3)
@@ -151,6 +151,7 @@ template <class T> struct DevSys {
     double* le_db;      // per replica: delta at the last list build (not reduced)
     int N;
     BondRec<T> bond;
+    T rc_max2;          // largest pair cutoff^2
     T rlist2;           // (rc + skin)^2
     T half_skin2;       // (skin / 2)^2
     T skin;
@@ -259,7 +260,7 @@ template <class T> struct Launch {
     // scratch); returns the number of kernels launched
     static int rebuild(const DevSys<T>& s, int cur, bool resort, bool permute_force, cudaStream_t st);
     // the list search of the replicas just binned (k_verlet.cu)
-    static void verlet(const DevSys<T>& s, cudaStream_t st);
+    static void verlet(const DevSys<T>& s, int cur, cudaStream_t st);
     static void request_all(const DevSys<T>& s, cudaStream_t st);
     // step kernels
     // one force evaluation (+ the learned potential's kernels); returns the

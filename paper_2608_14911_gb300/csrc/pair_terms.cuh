@@ -39,42 +39,42 @@ __device__ __forceinline__ void pair_force(const PairRec<T>& pr, const T* __rest
     u = pr.eps4 * s6 * (s6 - T(1)) - pr.shift;
 }
 
+// |F| / r of one pair at displacement d (0 beyond the cutoff); adds its energy and
+// virial.
+template <class T, bool ENERGY, bool MULTI, bool FAST>
+__device__ __forceinline__ T pair_scalar(const DevSys<T>& s, int ti, const PairRec<T>* pr1, T dx, T dz, T r2, int tj,
+                                         T& pe, T& vir, T& vxz) {
+    T fr, u;
+    if (FAST) {
+        // one type, plain Lennard-Jones: only rc^2, sigma^2, 24 eps live
+        if (!less_nonneg(r2, pr1->rc2)) return T(0);
+        const T inv_r2 = recip(r2);
+        const T s2 = pr1->sig2 * inv_r2;
+        const T s6 = s2 * s2 * s2;
+        fr = pr1->eps24 * s6 * (T(2) * s6 - T(1)) * inv_r2;
+        if (ENERGY) u = pr1->eps4 * s6 * (s6 - T(1)) - pr1->shift;
+    } else {
+        const PairRec<T>& pr = MULTI ? s.pair[ti * s.ntypes + tj] : *pr1;
+        if ((MULTI && pr.kind == 0) || !less_nonneg(r2, pr.rc2)) return T(0);
+        pair_force(pr, s.tab, r2, fr, u);
+    }
+    if (ENERGY) {
+        pe += u;
+        vir += fr * r2;
+        vxz += fr * dx * dz;
+    }
+    return fr;
+}
+
 // One pair term: force (and energy, virial) of neighbour j at displacement d.
 template <class T, bool ENERGY, bool MULTI, bool FAST>
 __device__ __forceinline__ void pair_term(const DevSys<T>& s, int ti, const PairRec<T>* pr1, T dx, T dy,
                                           T dz, int tj, T& fx, T& fy, T& fz, T& pe, T& vir, T& vxz) {
     const T r2 = dx * dx + dy * dy + dz * dz;
-    if (FAST) {
-        // one type, plain Lennard-Jones: only rc^2, sigma^2, 24 eps live
-        if (r2 < pr1->rc2) {
-            const T inv_r2 = recip(r2);
-            const T s2 = pr1->sig2 * inv_r2;
-            const T s6 = s2 * s2 * s2;
-            const T fr = pr1->eps24 * s6 * (T(2) * s6 - T(1)) * inv_r2;
-            fx += fr * dx;
-            fy += fr * dy;
-            fz += fr * dz;
-            if (ENERGY) {
-                pe += pr1->eps4 * s6 * (s6 - T(1)) - pr1->shift;
-                vir += fr * r2;
-                vxz += fr * dx * dz;
-            }
-        }
-        return;
-    }
-    const PairRec<T>& pr = MULTI ? s.pair[ti * s.ntypes + tj] : *pr1;
-    if ((!MULTI || pr.kind != 0) && r2 < pr.rc2) {
-        T fr, u;
-        pair_force(pr, s.tab, r2, fr, u);
-        fx += fr * dx;
-        fy += fr * dy;
-        fz += fr * dz;
-        if (ENERGY) {
-            pe += u;
-            vir += fr * r2;
-            vxz += fr * dx * dz;
-        }
-    }
+    const T fr = pair_scalar<T, ENERGY, MULTI, FAST>(s, ti, pr1, dx, dz, r2, tj, pe, vir, vxz);
+    fx += fr * dx;
+    fy += fr * dy;
+    fz += fr * dz;
 }
 
 // Lees-Edwards quantities of the current step, uniform over a tile: delta

@@ -25,10 +25,20 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
 
 // Top 24 bits k of a word -> (2k + 1 - 2^24) * 2^-25: an odd multiple of 2^-25
 // in (-1/2, 1/2), exact in float and double, mean 0, variance (1-2^-48)/12.
+// Formed in float (a 24-bit integer, a power of two: exact); doubles are widened
+// by moving the bits (the value is never zero, subnormal or infinite), which
+// spares the FP64 unit a conversion and a product.
 template <class T>
-__device__ __forceinline__ T uniform_centered(unsigned int w) {
+__device__ __forceinline__ T uniform_centered(unsigned int w);
+template <>
+__device__ __forceinline__ float uniform_centered<float>(unsigned int w) {
     const int odd = 2 * (int)(w >> 8) + 1 - 16777216;
-    return (T)odd * (T)2.98023223876953125e-08;
+    return (float)odd * 2.98023223876953125e-08f;
+}
+template <>
+__device__ __forceinline__ double uniform_centered<double>(unsigned int w) {
+    const unsigned int b = __float_as_uint(uniform_centered<float>(w));
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
 }
 
 // Langevin noise of one particle: key (seed lo, seed hi), counter

@@ -499,6 +499,8 @@ class System : public SystemBase {
         // the general step-kernel variants take
         d.lj_fast = (!d.cells_mode && ntypes == 1 && pair_h[0][0].kind == ESPP_LJ) ? 1 : 0;
         d.mlp_on = (pair_h[0][0].kind == ESPP_MLP) ? 1 : 0;
+        d.rc_max2 = T(0);
+        for (int k = 0; k < ntypes * ntypes; ++k) d.rc_max2 = std::max(d.rc_max2, pr[k].rc2);
         if (d.mlp_on && !mlp_bits.empty()) {
             MlpWeights w;
             memset(&w, 0, sizeof(w));
