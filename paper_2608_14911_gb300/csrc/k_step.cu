@@ -17,6 +17,7 @@
 // and checks the displacement since the last list build against skin/2.
 #include "kernels.cuh"
 #include "packed.cuh"
+#include "pair_queue.cuh"
 #include "pair_terms.cuh"
 #include "philox.cuh"
 
@@ -221,14 +222,6 @@ struct PairQueue {
     T th[DPD ? QR : 1];     // the thermostat's term
 };
 
-// a coordinate in FP32: FP64 ones are cut to 20 mantissa bits (|x| < 2^-126 to 0)
-__device__ __forceinline__ float cut(float x) { return x; }
-__device__ __forceinline__ float cut(double x) {
-    const int hi = __double2hiint(x);
-    const unsigned int a = max(hi & 0x7fffffff, 0x38000000) - 0x38000000;
-    return __uint_as_float((a << 3) | (hi & 0x80000000u));
-}
-
 // PPW: particles per warp, 32 (one lane each) or 8 (four lanes share a
 // particle: lane t takes entry t of every group).  Returns the pair force on the
 // lane's particle (PPW 8: on each of its four lanes); pe, vir, vxz: sums over the
@@ -306,26 +299,16 @@ __device__ __forceinline__ void queue_loop(const DevSys<T>& s, const V4<T>* __re
             }
         }
         // where each particle's terms start in the warp's queue
-        int off = t0 == 0 ? cnt : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_up_sync(0xffffffffu, off, o);
-            if (lane >= o) off += u;
-        }
-        const int total = __shfl_sync(0xffffffffu, off, 31);
-        if (t0 == 0) off -= cnt;
+        int total;
+        const int off = queue_offsets(t0 == 0 ? cnt : 0, total);
         const int from = TPP == 1 ? off : __shfl_sync(0xffffffffu, off, lane & 28), to = from + cnt;
         for (int r0 = 0; r0 < total; r0 += QR) {
             const int nr = min(QR, total - r0);
             __syncwarp();
             for (int b = 0; b < nr; b += 32) {
                 const int q = min(b + lane, nr - 1) + r0;
-                // the particle of entry q: the last lane whose terms start at or before q
-                int own = 0;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1)
-                    if (__shfl_sync(0xffffffffu, off, own + o) <= q) own += o;
-                const int k = q - __shfl_sync(0xffffffffu, off, own);
+                int k;
+                const int own = queue_owner(off, q, k);
                 if (b + lane < nr) {
                     const int p = TPP == 1 ? own : own >> 2;
                     const int e = Q.col[k * PPW + p];
@@ -368,29 +351,7 @@ __device__ __forceinline__ void queue_loop(const DevSys<T>& s, const V4<T>* __re
                 }
             }
             __syncwarp();
-            const int k0 = max(from, r0) - r0, k1 = min(to, r0 + nr) - r0;
-            if constexpr (TPP == 1) {
-                for (int k = k0; k < k1; ++k) {
-                    const T fr = Q.fr[k], dx = Q.dx[k], dy = Q.dy[k], dz = Q.dz[k];
-                    fx = fma_rn(fr, dx, fx);
-                    fy = fma_rn(fr, dy, fy);
-                    fz = fma_rn(fr, dz, fz);
-                    if (DPD) {
-                        const T th = Q.th[k];
-                        fx = fma_rn(th, dx, fx);
-                        fy = fma_rn(th, dy, fy);
-                        fz = fma_rn(th, dz, fz);
-                    }
-                }
-            } else {
-                // one component per lane
-                const T* d = t0 == 0 ? Q.dx : t0 == 1 ? Q.dy : Q.dz;
-                for (int k = k0; k < k1; ++k) {
-                    const T dd = d[k];
-                    fx = fma_rn(Q.fr[k], dd, fx);
-                    if (DPD) fx = fma_rn(Q.th[k], dd, fx);
-                }
-            }
+            queue_add<T, DPD, TPP>(Q, max(from, r0) - r0, min(to, r0 + nr) - r0, t0, fx, fy, fz);
         }
         __syncwarp();
     }

@@ -85,3 +85,37 @@ def test_spread_does_not_change_the_bits(prec, dpd, n):
         s.close()
     for a, b, both in zip(*out):
         assert np.array_equal(np.concatenate([a, b]), both)
+
+
+@pytest.mark.parametrize("prec,tol", [(FP32, 1e-5), (FP64, 1e-12)])
+@pytest.mark.parametrize("n,density", [(33, 0.3), (129, 0.8), (700, 6.0), (1500, 12.0)])
+def test_cell_forces(n, density, prec, tol):
+    # the list-free force kernel: partial warps, columns that fill inside a row
+    c = _gas(n, density, 8)
+    s = _handle([c], prec)
+    s.set_force_method(espp.ESPP_FORCES_CELLS)
+    f = s.compute_forces()
+    o = s.observables()
+    s.close()
+    m = O.Model(1, {(0, 0): CAP}, None)
+    fo, _ = O.forces(m, c.box, c.x, c.types, c.bonds)
+    assert rel_rms(f, fo) <= tol
+    oo = O.observables(m, O.State(c.box, c.x, c.v, c.img, c.types, c.bonds))
+    for k in ("pe_pair", "virial"):
+        assert abs(o[k] - oo[k]) <= tol * abs(oo[k]), k
+
+
+@pytest.mark.parametrize("prec", [FP32, FP64])
+def test_cell_forces_spread_does_not_change_the_bits(prec):
+    # each replica alone takes eight lanes per particle, both together one
+    cs = [_gas(22000, 0.7, seed) for seed in (3, 4)]
+    out = []
+    for group in ([cs[0]], [cs[1]], cs):
+        s = _handle(group, prec)
+        s.set_thermostat(espp.ESPP_THERMO_DPD, 1.1)
+        s.set_force_method(espp.ESPP_FORCES_CELLS)
+        s.integrate(6, 0.002, 1.0, 1.0)
+        out.append(s.get_state())
+        s.close()
+    for a, b, both in zip(*out):
+        assert np.array_equal(np.concatenate([a, b]), both)
