@@ -263,7 +263,12 @@ struct Ctrl {
                                // (inside an integrate call, after the first drift)
     unsigned int le_keep;      // the next rebuild keeps the stored Lees-Edwards build
                                // offsets (a checkpoint load), then clears this
-    unsigned int pad;
+    // resident run kernel (k_run.cu)
+    unsigned int bar;          // arrivals at its grid barrier
+    long long target;          // last step of the run's segment
+    long long stop;            // step after which a rebuild was requested or an error found
+    int final_step;            // the segment's last step ends the integrate call
+    int buf;                   // position buffer of step + 1 (read where a kernel gets buffer -1)
 };
 
 enum : unsigned int {

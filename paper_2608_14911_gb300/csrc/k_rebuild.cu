@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(TILE) k_bin(DevSys<T> s, int cur) {
         for (int r = threadIdx.x; r < s.R; r += blockDim.x) s.req[r] = 0;
         if (threadIdx.x == 0) s.ctrl->any_req = 0;
     }
-    V4<T>* __restrict__ P = s.pos[cur];
+    V4<T>* __restrict__ P = s.pos[buffer_of(s, cur)];
     for (int t = blockIdx.x; t < s.ntiles; t += gridDim.x) {
         const Tile tl = t == (int)blockIdx.x ? tl0 : s.tiles[t];
         if (!s.now[tl.rep] || (int)threadIdx.x >= tl.count) continue;
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(TILE) k_place(DevSys<T> s, int cur) {
     Tile tl0 = {0, 0, 0, 0};
     if ((int)blockIdx.x < s.ntiles) tl0 = ld_tile_early(s.tiles + blockIdx.x);
     if (s.ctrl->abort) return;
-    const V4<T>* __restrict__ P = s.pos[cur];
+    const V4<T>* __restrict__ P = s.pos[buffer_of(s, cur)];
     for (int t = blockIdx.x; t < s.ntiles; t += gridDim.x) {
         const Tile tl = t == (int)blockIdx.x ? tl0 : s.tiles[t];
         if (!s.now[tl.rep] || (int)threadIdx.x >= tl.count) continue;

@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? 8 : 6) k_verlet(DevSys<
         if (!s.now[tl.rep]) continue;  // uniform over the block
         VerletSearch<T, W, EXCL, LE, 1> v(s, s.reps[tl.rep]);
         v.EF = entries_f(s);
-        v.P = s.pos[cur];
+        v.P = sizeof(T) == 8 ? s.pos[buffer_of(s, cur)] : nullptr;  // (FP32 handles have no second test)
         v.col = buf[threadIdx.x >> 5] + (threadIdx.x & 31);
         v.sub = 0;
         v.tmask = 0;
@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(TILE, 6) k_verlet_team(DevSys<T> s, int cur) {
     if (q >= tl.count) return;   // whole teams
     VerletSearch<T, W, EXCL, LE, VTEAM> v(s, s.reps[tl.rep]);
     v.EF = entries_f(s);
-    v.P = s.pos[cur];
+    v.P = sizeof(T) == 8 ? s.pos[buffer_of(s, cur)] : nullptr;  // (FP32 handles have no second test)
     v.col = buf[team];
     v.sub = lane % VTEAM;
     v.tmask = ((1u << VTEAM) - 1u) << (lane / VTEAM * VTEAM);

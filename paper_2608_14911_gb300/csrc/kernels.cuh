@@ -243,6 +243,10 @@ __device__ __forceinline__ int cell_coord(T x, T cpl, int nc) {
 __device__ __forceinline__ const float4* entries_f(const DevSys<float>& s) { return s.cell_ent; }
 __device__ __forceinline__ const float4* entries_f(const DevSys<double>& s) { return s.cell_ent32; }
 
+// the position buffer of a rebuild kernel: given by the host, or (-1) the run's
+template <class T>
+__device__ __forceinline__ int buffer_of(const DevSys<T>& s, int cur) { return cur < 0 ? s.ctrl->buf : cur; }
+
 // kernels launched by one rebuild without a resort (Launch::rebuild)
 constexpr int REBUILD_LAUNCHES = 8;
 
@@ -267,6 +271,11 @@ template <class T> struct Launch {
     // number of kernels launched
     static int step(const DevSys<T>& s, int mode, bool energy, int cur, double* f_out,
                     unsigned long long next_cond, int grid, cudaStream_t st);
+    // resident run kernel: whether the handle's configuration takes it; the
+    // segment's parameters; the kernel itself (cond: the loop's condition)
+    static bool run_fits(const DevSys<T>& s);
+    static void run_begin(const DevSys<T>& s, long long target, int final_step, int buf, cudaStream_t st);
+    static cudaError_t run(const DevSys<T>& s, unsigned long long cond, cudaStream_t st);
     static void prologue(const DevSys<T>& s, int cur, int grid, cudaStream_t st);
     static void set_cond(const DevSys<T>& s, unsigned long long cond, cudaStream_t st);
     // the learned potential's pair forces: the tensor-core path (FP32 handles)

@@ -1337,6 +1337,56 @@ class System : public SystemBase {
         return ESPP_OK;
     }
 
+    // Small systems: one graph runs a whole segment of steps (k_run.cu): run,
+    // then, while steps are left, rebuild and run again.
+    bool use_run() const { return chunk > 0 && !timing && Launch<T>::run_fits(d); }
+    int make_run(ChunkGraph** out) {
+        auto key = std::make_tuple(0, 0, 0, 0);
+        auto it = graphs.find(key);
+        if (it != graphs.end()) {
+            *out = &it->second;
+            return ESPP_OK;
+        }
+        cudaStream_t cs = nullptr, bs = nullptr;
+        CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
+        CK(cudaStreamCreateWithFlags(&bs, cudaStreamNonBlocking));
+        cudaGraph_t g;
+        CK(cudaGraphCreate(&g, 0));
+        cudaGraphConditionalHandle h;
+        CK(cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault));
+        CK(cudaStreamBeginCaptureToGraph(cs, g, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
+        CK(Launch<T>::run(d, (unsigned long long)h, cs));
+        cudaStreamCaptureStatus status;
+        cudaGraph_t capg;
+        const cudaGraphNode_t* deps = nullptr;
+        size_t nd = 0;
+        CK(cudaStreamGetCaptureInfo(cs, &status, nullptr, &capg, &deps, nullptr, &nd));
+        alignas(cudaGraphNodeParams) unsigned char raw[sizeof(cudaGraphNodeParams)];
+        memset(raw, 0, sizeof(raw));
+        cudaGraphNodeParams& np = *reinterpret_cast<cudaGraphNodeParams*>(raw);
+        np.type = cudaGraphNodeTypeConditional;
+        np.conditional.handle = h;
+        np.conditional.type = cudaGraphCondTypeWhile;
+        np.conditional.size = 1;
+        cudaGraphNode_t node;
+        CK(cudaGraphAddNode(&node, capg, deps, nullptr, nd, &np));
+        cudaGraph_t body = np.conditional.phGraph_out[0];
+        CK(cudaStreamUpdateCaptureDependencies(cs, &node, nullptr, 1, cudaStreamSetCaptureDependencies));
+        CK(cudaStreamBeginCaptureToGraph(bs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
+        Launch<T>::rebuild(d, -1, false, false, bs);
+        CK(Launch<T>::run(d, (unsigned long long)h, bs));
+        cudaGraph_t tmp, done;
+        CK(cudaStreamEndCapture(bs, &tmp));
+        CK(cudaStreamEndCapture(cs, &done));
+        ChunkGraph cg;
+        CK(cudaGraphInstantiate(&cg.exec, done, 0));
+        cudaStreamDestroy(cs);
+        cudaStreamDestroy(bs);
+        cg.graph = done;
+        *out = &graphs.emplace(key, std::move(cg)).first->second;
+        return ESPP_OK;
+    }
+
     // timing mode: add the event-measured durations of the last replay of a chunk
     int harvest_timing(ChunkGraph* cg) {
         const size_t S = cg->ev.size() / 3;
@@ -1394,6 +1444,10 @@ class System : public SystemBase {
     // after the first one on a configuration launch cached graphs only.
     int prepare_graphs() {
         if (chunk <= 0) return ESPP_OK;
+        if (use_run()) {
+            ChunkGraph* cg = nullptr;
+            return make_run(&cg);
+        }
         for (int p = 0; p < 2; ++p) {
             ChunkGraph* cg = nullptr;
             for (int S : chunk_sizes()) {
@@ -1446,6 +1500,7 @@ class System : public SystemBase {
             int p = (1 - c_start) ^ (int)((done - step0) & 1);
             int64_t next = done + 1;  // step the next graph computes first
             int64_t host_rebuilds = 0;  // rebuilds launched here rather than by graph nodes
+            bool runs = false;          // the resident run kernel, launched again after each rebuild
             while (next <= target) {
                 // Hilbert resort (with a list rebuild) before every step that is
                 // a multiple of resort_every: a function of the step number only
@@ -1453,6 +1508,22 @@ class System : public SystemBase {
                     Launch<T>::request_all(d, st);
                     launches += 1 + Launch<T>::rebuild(d, p, true, false, st);
                     host_rebuilds++;
+                }
+                if (use_run()) {
+                    // the whole segment up to the next resort or the call's end
+                    int64_t S = target - next + 1;
+                    if (resort_every > 0) S = std::min<int64_t>(S, resort_every - (next % resort_every));
+                    const bool ends = next + S - 1 == target;
+                    ChunkGraph* cg = nullptr;
+                    rcode = make_run(&cg);
+                    if (rcode) return rcode;
+                    Launch<T>::run_begin(d, next + S - 1, ends ? 1 : 0, p, st);
+                    CK(cudaGraphLaunch(cg->exec, st));
+                    launches += 2;
+                    p ^= (int)((S - (ends ? 1 : 0)) & 1);
+                    next += S;
+                    runs = true;
+                    continue;
                 }
                 // steps before the final one, up to the next resort
                 int64_t avail = target - next;
@@ -1490,7 +1561,7 @@ class System : public SystemBase {
             Ctrl c = read_ctrl();
             CK(cudaGetLastError());
             if (host_rebuilds >= 0)
-                launches += (REBUILD_LAUNCHES - (d.cells_mode ? 1 : 0) + (d.mlp_on ? 5 : 0)) *
+                launches += (REBUILD_LAUNCHES - (d.cells_mode ? 1 : 0) + (d.mlp_on ? 5 : 0) + (runs ? 1 : 0)) *
                             ((int64_t)(c.n_rebuilds - (unsigned)rb0) - host_rebuilds);
             if (c.err & (ERRBIT_BOND | ERRBIT_NONFINITE | ERRBIT_TIMEOUT)) return status_from(c);
             if (c.err & ERRBIT_OVERFLOW) {

@@ -1,0 +1,65 @@
+"""The resident run kernel (small systems: many steps in one launch) against the
+same steps launched one kernel at a time: the same bits, at the sizes where
+its forms change and across list rebuilds, Hilbert resorts and calls of odd
+lengths; and a run it cannot finish reports what stopped it."""
+import numpy as np
+import pytest
+
+from paper_2608_14911_gb300 import espp, inputs as I
+
+from _systems import WCA_RC
+
+pytestmark = pytest.mark.gpu
+FP32, FP64 = espp.ESPP_FP32, espp.ESPP_FP64
+
+
+def _melt(chains, beads, prec, chunk=None):
+    c = I.kg_lattice(chains, beads, density=0.85, seed=4)
+    s = espp.System(c.box, c.n, c.types, c.bonds, precision=prec, seed=4)
+    s.set_wca()
+    s.set_fene()
+    if chunk is not None:
+        s.set_graph_chunk(chunk)
+    s.set_resort_interval(20)
+    s.set_state(c.x, I.maxwell_velocities(c.n, 1.0, seed=4), c.img)
+    s.build_neighbors(WCA_RC, 0.4)
+    return s
+
+
+@pytest.mark.parametrize("prec,chains,beads", [
+    (FP32, 3, 43),        # a partial tile (129)
+    (FP32, 40, 100),
+    (FP32, 304, 128),     # the last size with 16 entries in flight
+    (FP32, 305, 128),     # and the next
+    (FP64, 3, 43),
+    (FP64, 114, 128),     # the last size with four lanes per particle
+    (FP64, 115, 128),
+])
+def test_run_equals_single_launches(prec, chains, beads):
+    a, b = _melt(chains, beads, prec), _melt(chains, beads, prec, chunk=0)
+    for n in (1, 2, 19, 33):
+        a.integrate(n, 0.005, 1.0, 1.0)
+        b.integrate(n, 0.005, 1.0, 1.0)
+        assert a.step == b.step and a.n_rebuilds == b.n_rebuilds
+        for p, q in zip(a.get_state(), b.get_state()):
+            assert np.array_equal(p, q)
+    assert a.n_rebuilds > 4
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("prec", [FP32, FP64])
+def test_broken_bond_stops_the_run(prec):
+    # a bond pulled past R0 by its beads' velocities, some steps into the run
+    s = _melt(20, 50, prec)
+    x, v, img = s.get_state()
+    v[0], v[1] = (-30.0, 0.0, 0.0), (30.0, 0.0, 0.0)
+    s.set_state(x, v, img)
+    with pytest.raises(espp.EsppError) as e:
+        s.integrate(200, 0.005, 0.0, 0.0)
+    assert e.value.code in (espp.ESPP_ERR_BOND_BROKEN, espp.ESPP_ERR_NONFINITE)
+    assert s.step < 200
+    # a new state clears the error, and the handle runs again
+    s.set_state(x, np.zeros_like(v), img)
+    s.integrate(5, 0.001, 1.0, 0.1)
+    s.close()
