@@ -14,36 +14,10 @@
 // potential, bonds and the Langevin thermostat, as long as one round of blocks
 // holds every particle (see run_fits); the arithmetic is the step kernel's, so the
 // trajectories are the same bits.
+#include "grid_barrier.cuh"
 #include "pair_walk.cuh"
 
 namespace espp {
-
-constexpr int RUN_WAIT = 1 << 21;  // polls of the barrier before giving up (a second or so)
-
-// Grid barrier number `phase` (1, 2, ..) of this launch; false if the wait ran out
-// (the error is recorded and the block leaves).  *stop receives the stopping step.
-__device__ __forceinline__ bool run_barrier(Ctrl* c, unsigned int phase, long long* sh) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned int goal = gridDim.x * phase;
-        atomicAdd(&c->bar, 1u);
-        unsigned int seen = 0;
-        int it = 0;
-        do {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&c->bar) : "memory");
-        } while (seen < goal && ++it < RUN_WAIT);
-        __threadfence();
-        sh[0] = *(volatile long long*)&c->stop;
-        sh[1] = seen >= goal;
-        if (seen < goal) {
-            atomicOr(&c->err, ERRBIT_TIMEOUT);
-            c->abort = 1;
-        }
-    }
-    __syncthreads();
-    return sh[1] != 0;
-}
 
 // PPW: particles per warp (FP64 handles: the pair queue; FP32: one lane each);
 // GB: list groups per batch (FP32); MINB: resident blocks per SM.
@@ -52,7 +26,7 @@ __global__ void __launch_bounds__(TILE, MINB) k_run(DevSys<T> s, unsigned long l
     constexpr bool QUEUE = sizeof(T) == 8;
     constexpr int TPP = 32 / PPW;  // lanes per particle, blocks per tile
     __shared__ __align__(16) unsigned char queue_mem[QUEUE ? sizeof(PairQueue<T, false, PPW>) * (TILE / 32) : 16];
-    __shared__ long long sh[2];
+    __shared__ long long stopped;
     Ctrl* c = s.ctrl;
     // what every block sees before any block can change it
     const long long step0 = *(volatile long long*)&c->step, target = c->target;
@@ -61,7 +35,7 @@ __global__ void __launch_bounds__(TILE, MINB) k_run(DevSys<T> s, unsigned long l
     const bool go = *(volatile unsigned int*)&c->abort == 0 && *(volatile unsigned int*)&c->any_req == 0 &&
                     step0 < target;
     unsigned int phase = 1;
-    bool ok = run_barrier(c, phase++, sh);
+    bool ok = grid_barrier(c, phase++, [] {});
     long long step = step0;
     if (ok && go) {
         const int lt = TPP > 1 ? (int)(blockIdx.x % TPP) * (TILE / TPP) + (int)threadIdx.x / TPP : (int)threadIdx.x;
@@ -151,28 +125,21 @@ __global__ void __launch_bounds__(TILE, MINB) k_run(DevSys<T> s, unsigned long l
                 xi.y = __shfl_sync(0xffffffffu, xi.y, threadIdx.x & 28);
                 xi.z = __shfl_sync(0xffffffffu, xi.z, threadIdx.x & 28);
             }
-            ok = run_barrier(c, phase++, sh);
-            if (!ok || step == target || sh[0] == step) break;
+            ok = grid_barrier(c, phase++, [&] { stopped = *(volatile long long*)&c->stop; });
+            if (!ok || step == target || stopped == step) break;
         }
         if (lead) s.vel[i] = v;
     }
     // the last block to leave hands over to the graph
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    grid_leave(c, [&] {
+        c->step = step;
+        c->buf = buf;
+        if (fin && step == target) c->pos_ahead = 0;
+        c->stop = -1;
         __threadfence();
-        if (atomicAdd(&c->blocks_done, 1u) == gridDim.x - 1) {
-            __threadfence();
-            c->step = step;
-            c->buf = buf;
-            if (fin && step == target) c->pos_ahead = 0;
-            c->bar = 0;
-            c->blocks_done = 0;
-            c->stop = -1;
-            __threadfence();
-            const bool more = step < target && *(volatile unsigned int*)&c->abort == 0;
-            if (cond) cudaGraphSetConditional(cond, more ? 1u : 0u);
-        }
-    }
+        const bool more = step < target && *(volatile unsigned int*)&c->abort == 0;
+        if (cond) cudaGraphSetConditional(cond, more ? 1u : 0u);
+    });
 }
 
 template <class T>

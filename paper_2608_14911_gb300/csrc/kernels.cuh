@@ -69,7 +69,7 @@ template <class T> struct DevSys {
     int* slot_of_id;    // global id -> storage slot
     int* perm;          // new slot -> old slot (rebuild)
     int* cellh;         // per old slot: global cell rank
-    int* in_cell;       // per old slot: arrival index in its cell
+    int* in_cell;       // per old slot: arrival index in its cell, then its rank there
     // Verlet list in groups of four: entry k of particle i sits at
     // nbr[4 * ((k / 4) * stride + i) + k % 4]; k < nbr_cnt[i] <= cap; the last
     // group is padded with nbr_pad, the slot after the last particle, whose
@@ -81,13 +81,14 @@ template <class T> struct DevSys {
     int stride;
     int nbr_pad;
     // cells, all replicas concatenated; cell index cell_off + (cz * ny + cy) * nx + cx
-    int* cell_cnt;
+    int* cell_cnt;      // zero between builds
+    int* cell_slot;     // storage slots by cell, in order of arrival
     // compact entries (position, storage slot in the w lane): those of cell h
     // are cell_ent[cell_beg[h] .. cell_beg[h + 1]), ascending slot
     V4<T>* cell_ent;
     float4* cell_ent32;     // FP64 handles: the entries in FP32 (list search)
     int* cell_beg;          // ncells + 1; cell_beg[ncells] = N
-    int* rank_start;        // first new slot of each cell in Hilbert-rank order (resort only)
+    int* rank_start;        // first new slot of each cell (resort only)
     int cell_w;             // cell subdivision: cells of edge >= (rc + skin) / cell_w (1, 2 or 3)
     const int* cell_by_rank;  // global Hilbert rank -> cell index
     const int* cell_rep;
@@ -247,9 +248,6 @@ __device__ __forceinline__ const float4* entries_f(const DevSys<double>& s) { re
 template <class T>
 __device__ __forceinline__ int buffer_of(const DevSys<T>& s, int cur) { return cur < 0 ? s.ctrl->buf : cur; }
 
-// kernels launched by one rebuild without a resort (Launch::rebuild)
-constexpr int REBUILD_LAUNCHES = 8;
-
 // step-kernel modes
 enum : int {
     MODE_FORCES = 0,  // conservative forces only, written to an id-ordered double buffer
@@ -258,11 +256,15 @@ enum : int {
     MODE_FINAL = 3,   // F_s, v_s stored (end of an integrate call)
 };
 
+int binning_blocks();
+
 // ---- launchers (defined in the .cu files) ----------------------------------
 template <class T> struct Launch {
     // rebuild pipeline on the positions in buffer `cur` (other buffer is
     // scratch); returns the number of kernels launched
     static int rebuild(const DevSys<T>& s, int cur, bool resort, bool permute_force, cudaStream_t st);
+    // kernels launched by the binning of one rebuild
+    static int binning_launches(const DevSys<T>& s);
     // the list search of the replicas just binned (k_verlet.cu)
     static void verlet(const DevSys<T>& s, int cur, cudaStream_t st);
     static void request_all(const DevSys<T>& s, cudaStream_t st);

@@ -313,7 +313,7 @@ class System : public SystemBase {
             (rc = alloc(&d.frc, n, allocs)) || (rc = alloc(&d.frc_alt, n, allocs)) ||
             (rc = alloc(&d.xb, n, allocs)) || (rc = alloc(&d.img, n, allocs)) ||
             (rc = alloc(&d.img_alt, n, allocs)) || (rc = alloc(&d.bond_slot, n, allocs)) ||
-            (rc = alloc(&d.cell_ent, n + ENTRY_PAD, allocs)) ||
+            (rc = alloc(&d.cell_ent, n + ENTRY_PAD, allocs)) || (rc = alloc(&d.cell_slot, n, allocs)) ||
             (sizeof(T) == 8 && (rc = alloc(&d.cell_ent32, n + ENTRY_PAD, allocs))))
             return rc;
         int2* bg = nullptr;
@@ -1113,12 +1113,11 @@ class System : public SystemBase {
         d.nscan_blocks = scan_blocks_for(C);
         if ((rc2 = alloc(&cnt, C, cell_allocs)) || (rc2 = alloc(&beg, C + 1, cell_allocs)) ||
             (rc2 = alloc(&rstart, C, cell_allocs)) || (rc2 = alloc(&crep, C, cell_allocs)) ||
-            (rc2 = alloc(&cbr, C, cell_allocs)) || (rc2 = alloc(&part, d.nscan_blocks, cell_allocs)))
+            (rc2 = alloc(&cbr, C, cell_allocs)) || (rc2 = alloc(&part, std::max(d.nscan_blocks, binning_blocks()), cell_allocs)))
             return rc2;
         CK(cudaMemcpy(crep, rep_of.data(), C * sizeof(int), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(cbr, by_rank.data(), C * sizeof(int), cudaMemcpyHostToDevice));
-        // every count starts at zero (a replica's counts sum to its particle
-        // count after its first build); the entry array ends at N
+        // every count starts at zero; the entry array ends at N
         CK(cudaMemset(cnt, 0, C * sizeof(int)));
         const int nn = (int)N;
         CK(cudaMemcpy(beg + C, &nn, sizeof(int), cudaMemcpyHostToDevice));
@@ -1290,12 +1289,18 @@ class System : public SystemBase {
         cudaGraph_t g;
         CK(cudaGraphCreate(&g, 0));
         std::vector<cudaGraphConditionalHandle> h(S);
-        for (int r = 0; r < S; ++r) CK(cudaGraphConditionalHandleCreate(&h[r], g, 0, cudaGraphCondAssignDefault));
+        if (!d.cells_mode)
+            for (int r = 0; r < S; ++r) CK(cudaGraphConditionalHandleCreate(&h[r], g, 0, cudaGraphCondAssignDefault));
         CK(cudaStreamBeginCaptureToGraph(cs, g, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
-        Launch<T>::set_cond(d, h[0], cs);
+        if (!d.cells_mode) Launch<T>::set_cond(d, h[0], cs);
         int p = p0;
         for (int r = 0; r < S; ++r) {
             if (timing) CK(cudaEventRecordWithFlags(cg.ev[3 * r], cs, cudaEventRecordExternal));
+            if (d.cells_mode) {
+                // list-free mode: every step is binned, without a gate (8 us of a
+                // step of 24,000 particles)
+                Launch<T>::rebuild(d, p, false, false, cs);
+            } else {
             cudaStreamCaptureStatus status;
             cudaGraph_t capg;
             const cudaGraphNode_t* deps = nullptr;
@@ -1317,10 +1322,12 @@ class System : public SystemBase {
             Launch<T>::rebuild(d, p, false, false, bs);
             cudaGraph_t tmp;
             CK(cudaStreamEndCapture(bs, &tmp));
+            }
             const bool last = r == S - 1;
             const int mode = (final_chunk && last) ? MODE_FINAL : MODE_STEP;
             if (timing) CK(cudaEventRecordWithFlags(cg.ev[3 * r + 1], cs, cudaEventRecordExternal));
-            Launch<T>::step(d, mode, false, p, nullptr, last ? 0ull : (unsigned long long)h[r + 1], 0, cs);
+            Launch<T>::step(d, mode, false, p, nullptr,
+                            last || d.cells_mode ? 0ull : (unsigned long long)h[r + 1], 0, cs);
             if (timing) CK(cudaEventRecordWithFlags(cg.ev[3 * r + 2], cs, cudaEventRecordExternal));
             if (mode == MODE_STEP) p ^= 1;
         }
@@ -1561,7 +1568,7 @@ class System : public SystemBase {
             Ctrl c = read_ctrl();
             CK(cudaGetLastError());
             if (host_rebuilds >= 0)
-                launches += (REBUILD_LAUNCHES - (d.cells_mode ? 1 : 0) + (d.mlp_on ? 5 : 0) + (runs ? 1 : 0)) *
+                launches += (Launch<T>::binning_launches(d) + (d.cells_mode ? 0 : 1) + (d.mlp_on ? 5 : 0) + (runs ? 1 : 0)) *
                             ((int64_t)(c.n_rebuilds - (unsigned)rb0) - host_rebuilds);
             if (c.err & (ERRBIT_BOND | ERRBIT_NONFINITE | ERRBIT_TIMEOUT)) return status_from(c);
             if (c.err & ERRBIT_OVERFLOW) {
