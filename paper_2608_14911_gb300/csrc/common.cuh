@@ -109,6 +109,17 @@ __device__ __forceinline__ bool positive(double a) {
 __device__ __forceinline__ bool negative(float a) { return a < 0.f; }
 __device__ __forceinline__ bool negative(double a) { return __double2hiint(a) < 0; }
 
+// A float as a double by moving its bits (a conversion occupies the FP64 unit);
+// zeros, subnormals, infinities and NaNs take the conversion.
+// (The conversion is a call: inlined, it runs for every value and is selected away.)
+__device__ __noinline__ inline double widen_converted(float f) { return (double)f; }
+__device__ __forceinline__ double widen(float f) {
+    const unsigned int u = __float_as_uint(f), e = u & 0x7f800000u;
+    if (e == 0u || e == 0x7f800000u) return u == 0u ? 0.0 : widen_converted(f);
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double d) { return d; }
+
 // ---------------------------------------------------------------------------
 // Minimum image of xi - xj for coordinates stored in [0, L).  The periodic
 // shift is applied to the larger coordinate first; that subtraction is exact

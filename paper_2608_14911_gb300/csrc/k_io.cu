@@ -32,11 +32,17 @@ __global__ void __launch_bounds__(TILE) k_set_state(DevSys<T> s, const double* _
                 bad = true;
                 xd = 0.0;
             }
-            const double fl = floor(xd / L);
-            double w = xd - fl * L;
-            int k = (int)fl + (img ? img[3 * (size_t)i + d] : 0);
-            if (w < 0.0) { w += L; k -= 1; }
-            if (w >= L) { w -= L; k += 1; }
+            double w = xd;
+            int k = img ? img[3 * (size_t)i + d] : 0;
+            // a coordinate inside the box, the common case, needs none of the
+            // FP64 work (1M particles: 116 us with it)
+            if (!(__double2hiint(xd) >= 0 && less_nonneg(xd, L))) {
+                const double fl = floor(xd / L);
+                w = xd - fl * L;
+                k += (int)fl;
+                if (w < 0.0) { w += L; k -= 1; }
+                if (w >= L) { w -= L; k += 1; }
+            }
             T wt = (T)w;
             if (wt >= g.L[d]) { wt = T(0); k += 1; }
             p[d] = wt;
@@ -69,16 +75,18 @@ __global__ void __launch_bounds__(TILE) k_get_state(DevSys<T> s, double* __restr
         const Tile tl = s.tiles[t];
         if ((int)threadIdx.x >= tl.count) continue;
         const RepGeom<T>& g = s.reps[tl.rep];
-        const int i = tl.start + threadIdx.x;
+        // by id: the arrays are written in order and the records gathered (a
+        // replica's ids and slots fill the same range)
+        const size_t gid = (size_t)tl.start + threadIdx.x;
+        const int i = s.slot_of_id[gid];
         const V4<T> vv = s.vel[i];
-        const size_t gid = (size_t)g.p_off + bits_as_int(vv.w);
         // stored positions may lie just outside the box (they are wrapped at
         // list builds only): report them wrapped, with the image counters to match
         const V4<T> p = s.pos[cur][i];
-        const double pc[3] = {(double)p.x, (double)p.y, (double)p.z};
+        const double pc[3] = {widen(p.x), widen(p.y), widen(p.z)};
         double wc[3];
         int sh[3];
-        double vx = (double)vv.x;
+        double vx = widen(vv.x);
         if (s.le_on) {
             // Lees-Edwards: a crossing of a sheared face also moves x and v_x
             const double L[3] = {(double)g.L[0], (double)g.L[1], (double)g.L[2]};
@@ -91,8 +99,8 @@ __global__ void __launch_bounds__(TILE) k_get_state(DevSys<T> s, double* __restr
                 const double L = (double)g.L[d];
                 double w = pc[d];
                 int k = 0;
-                if (w >= L) { w -= L; k = 1; }
-                else if (w < 0.0) {
+                if (!(__double2hiint(w) >= 0 && less_nonneg(w, L)) && w >= L) { w -= L; k = 1; }
+                else if (__double2hiint(w) < 0 && w < 0.0) {
                     w += L;
                     k = -1;
                     if (w >= L) { w = 0.0; k = 0; }  // less than half an ulp below 0: its own image
@@ -108,8 +116,8 @@ __global__ void __launch_bounds__(TILE) k_get_state(DevSys<T> s, double* __restr
         }
         if (v) {
             v[3 * gid] = vx;
-            v[3 * gid + 1] = vv.y;
-            v[3 * gid + 2] = vv.z;
+            v[3 * gid + 1] = widen(vv.y);
+            v[3 * gid + 2] = widen(vv.z);
         }
         if (img) {
             const int4 im = s.img[i];
@@ -119,9 +127,9 @@ __global__ void __launch_bounds__(TILE) k_get_state(DevSys<T> s, double* __restr
         }
         if (f) {
             const V4<T> fi = s.frc[i];
-            f[3 * gid] = fi.x;
-            f[3 * gid + 1] = fi.y;
-            f[3 * gid + 2] = fi.z;
+            f[3 * gid] = widen(fi.x);
+            f[3 * gid + 1] = widen(fi.y);
+            f[3 * gid + 2] = widen(fi.z);
         }
     }
 }
@@ -139,71 +147,108 @@ __global__ void __launch_bounds__(TILE) k_set_force(DevSys<T> s, const double* _
     }
 }
 
-// One block per replica sums its tiles' partials in a fixed order.
+// One block per replica and quantity sums its tiles' partials in a fixed order
+// (one quantity after the other in one block: 27 us for 1563 tiles).
 template <class T>
 __global__ void __launch_bounds__(256) k_reduce_obs(DevSys<T> s, double* __restrict__ out) {
-    const int r = blockIdx.x;
+    const int r = blockIdx.x, k = blockIdx.y;
     const int t0 = s.rep_tile_off[r], t1 = s.rep_tile_off[r + 1];
     __shared__ double sh[256];
-    for (int k = 0; k < NPART; ++k) {
-        double a = 0.0;
-        for (int t = t0 + threadIdx.x; t < t1; t += blockDim.x) a += s.partials[(size_t)t * NPART + k];
-        sh[threadIdx.x] = a;
-        __syncthreads();
-        for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-            if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) out[(size_t)r * NPART + k] = sh[0];
+    double a = 0.0;
+    for (int t = t0 + threadIdx.x; t < t1; t += blockDim.x) a += s.partials[(size_t)t * NPART + k];
+    sh[threadIdx.x] = a;
+    __syncthreads();
+    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
         __syncthreads();
     }
+    if (threadIdx.x == 0) out[(size_t)r * NPART + k] = sh[0];
 }
 
 // One warp per molecule: centre of the unwrapped positions, then the mean
-// squared distance from it, both summed in a fixed lane order.
+// squared distance from it, both summed in a fixed lane order.  FP64 work bounds
+// it (four warps per molecule: 36 us instead of 25 for 1000 chains of 200 beads),
+// so the positions of chains of up to 256 beads are converted once and kept.
 template <class T>
 __global__ void k_rg2(DevSys<T> s, int cur, const int* __restrict__ members,
                       const int* __restrict__ off, const int* __restrict__ mrep, int nmol,
                       double* __restrict__ rg2) {
+    constexpr int KEEP = 8;
     const int lane = threadIdx.x & 31;
     const int m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (m >= nmol) return;
     const RepGeom<T>& g = s.reps[mrep[m]];
     const int b = off[m], e = off[m + 1];
+    const double L0 = (double)g.L[0], L1 = (double)g.L[1], L2 = (double)g.L[2];
     // Lees-Edwards: the unwrapped x adds img_z delta(t) (delta not reduced)
     const double dle = s.le_on ? le_offset(s, g, s.ctrl->step + (long long)s.ctrl->pos_ahead) : 0.0;
-    double c[3] = {0.0, 0.0, 0.0};
-    for (int k = b + lane; k < e; k += 32) {
+    auto unwrapped = [&](int k, double u[3]) {
         const int slot = s.slot_of_id[members[k]];
         const V4<T> p = s.pos[cur][slot];
         const int4 im = s.img[slot];
-        c[0] += (double)p.x + (double)im.x * (double)g.L[0] + (double)im.z * dle;
-        c[1] += (double)p.y + (double)im.y * (double)g.L[1];
-        c[2] += (double)p.z + (double)im.z * (double)g.L[2];
+        u[0] = widen(p.x);
+        u[1] = widen(p.y);
+        u[2] = widen(p.z);
+        if (im.x) u[0] += (double)im.x * L0;
+        if (im.y) u[1] += (double)im.y * L1;
+        if (im.z) {
+            u[0] += (double)im.z * dle;
+            u[2] += (double)im.z * L2;
+        }
+    };
+    double c[3] = {0.0, 0.0, 0.0}, kept[KEEP][3];
+#pragma unroll
+    for (int q = 0; q < KEEP; ++q) {
+        const int k = b + lane + 32 * q;
+        if (k >= e) continue;
+        unwrapped(k, kept[q]);
+        for (int d = 0; d < 3; ++d) c[d] += kept[q][d];
+    }
+    double u[3];
+    for (int k = b + lane + 32 * KEEP; k < e; k += 32) {
+        unwrapped(k, u);
+        for (int d = 0; d < 3; ++d) c[d] += u[d];
     }
     for (int d = 0; d < 3; ++d) {
         for (int o = 16; o > 0; o >>= 1) c[d] += __shfl_xor_sync(0xffffffffu, c[d], o);
         c[d] /= (double)(e - b);
     }
     double a = 0.0;
-    for (int k = b + lane; k < e; k += 32) {
-        const int slot = s.slot_of_id[members[k]];
-        const V4<T> p = s.pos[cur][slot];
-        const int4 im = s.img[slot];
-        const double ux = (double)p.x + (double)im.x * (double)g.L[0] + (double)im.z * dle - c[0];
-        const double uy = (double)p.y + (double)im.y * (double)g.L[1] - c[1];
-        const double uz = (double)p.z + (double)im.z * (double)g.L[2] - c[2];
+    auto add = [&](const double v[3]) {
+        const double ux = v[0] - c[0], uy = v[1] - c[1], uz = v[2] - c[2];
         a += ux * ux + uy * uy + uz * uz;
+    };
+#pragma unroll
+    for (int q = 0; q < KEEP; ++q)
+        if (b + lane + 32 * q < e) add(kept[q]);
+    for (int k = b + lane + 32 * KEEP; k < e; k += 32) {
+        unwrapped(k, u);
+        add(u);
     }
     for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
     if (lane == 0) rg2[m] = a / (double)(e - b);
+}
+
+// Histogram bin of a distance: (int)(sqrt(r2) * inv_dr) in double.  The FP32 value
+// decides wherever it lies further from a bin edge than its error (three
+// roundings, under 4e-7 of it); the FP64 root is taken near the edges only.
+// (a function of its own: inlined, its FP64 root runs for every pair and a select
+// drops it)
+__device__ __noinline__ int rdf_bin_exact(double r2, double inv_dr) { return (int)(sqrt(r2) * inv_dr); }
+template <class T>
+__device__ __forceinline__ int rdf_bin(T r2, double inv_dr, float inv_drf, int nbins) {
+    const float x = sqrtf((float)r2) * inv_drf;
+    const float lo = floorf(x), m = 4e-7f * x + 1e-30f;
+    int b = (int)lo;
+    if (x - lo <= m || lo + 1.f - x <= m) b = rdf_bin_exact((double)r2, inv_dr);
+    return b >= nbins ? nbins - 1 : b;
 }
 
 // Unique pairs (slot i < slot j) of one replica with r < rmax; integer bin
 // counts (exact under atomics).
 template <class T>
 __global__ void __launch_bounds__(256) k_rdf(DevSys<T> s, int cur, int rep, T rmax2, double inv_dr,
-                                             int nbins, unsigned long long* __restrict__ counts) {
+                                             float inv_drf, int nbins, unsigned long long* __restrict__ counts) {
     extern __shared__ unsigned int hist[];
     for (int b = threadIdx.x; b < nbins; b += blockDim.x) hist[b] = 0;
     __syncthreads();
@@ -224,9 +269,7 @@ __global__ void __launch_bounds__(256) k_rdf(DevSys<T> s, int cur, int rep, T rm
                          : min_image(a.x, c.x, g.L[0], g.halfL[0]);
         const T r2 = dx * dx + dy * dy + dz * dz;
         if (r2 < rmax2) {
-            int b = (int)(sqrt((double)r2) * inv_dr);
-            if (b >= nbins) b = nbins - 1;
-            atomicAdd(&hist[b], 1u);
+            atomicAdd(&hist[rdf_bin(r2, inv_dr, inv_drf, nbins)], 1u);
         }
       }
     __syncthreads();
@@ -237,8 +280,8 @@ __global__ void __launch_bounds__(256) k_rdf(DevSys<T> s, int cur, int rep, T rm
 // Unique pairs within rmax from the Verlet list (rmax <= list cutoff): each
 // pair appears in both lists, counted from the lower storage slot.
 template <class T>
-__global__ void __launch_bounds__(256) k_rdf_list(DevSys<T> s, int cur, int rep, T rmax2, double inv_dr, int nbins,
-                                                  unsigned long long* __restrict__ counts) {
+__global__ void __launch_bounds__(256) k_rdf_list(DevSys<T> s, int cur, int rep, T rmax2, double inv_dr,
+                                                  float inv_drf, int nbins, unsigned long long* __restrict__ counts) {
     extern __shared__ unsigned int hist[];
     for (int b = threadIdx.x; b < nbins; b += blockDim.x) hist[b] = 0;
     __syncthreads();
@@ -252,21 +295,27 @@ __global__ void __launch_bounds__(256) k_rdf_list(DevSys<T> s, int cur, int rep,
         const int i = g.p_off + q;
         const V4<T> xi = P[i];
         const int n = s.nbr_cnt[i];
-        for (int k = 0; k < n; ++k) {
-            const int e = s.nbr[4 * ((size_t)(k >> 2) * stride + i) + (k & 3)];
-            const int j = nbr_slot(e);
-            if (j < i) continue;
-            const V4<T> xj = P[j];
-            const int code = nbr_code(e);
-            const T dx = (code & 3) == 3 ? le_dx(xi.x, xj.x, (code >> 4) == 1 ? 1 : -1, dle, g.L[0], T(1) / g.L[0])
-                                         : shifted_diff(xi.x, xi.x - g.L[0], xj.x, g.L[0], code & 3);
-            const T dy = shifted_diff(xi.y, xi.y - g.L[1], xj.y, g.L[1], (code >> 2) & 3);
-            const T dz = shifted_diff(xi.z, xi.z - g.L[2], xj.z, g.L[2], code >> 4);
-            const T r2 = dx * dx + dy * dy + dz * dz;
-            if (r2 < rmax2) {
-                int b = (int)(sqrt((double)r2) * inv_dr);
-                if (b >= nbins) b = nbins - 1;
-                atomicAdd(&hist[b], 1u);
+        for (int k0 = 0; k0 < n; k0 += 4) {
+            const int4 grp = reinterpret_cast<const int4*>(s.nbr)[(size_t)(k0 >> 2) * stride + i];
+            const int en[4] = {grp.x, grp.y, grp.z, grp.w};
+            V4<T> xj[4];
+            bool own[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                own[q] = k0 + q < n && nbr_slot(en[q]) > i;
+                if (own[q]) xj[q] = P[nbr_slot(en[q])];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (!own[q]) continue;
+                const int code = nbr_code(en[q]);
+                const T dx = (code & 3) == 3
+                                 ? le_dx(xi.x, xj[q].x, (code >> 4) == 1 ? 1 : -1, dle, g.L[0], T(1) / g.L[0])
+                                 : shifted_diff(xi.x, xi.x - g.L[0], xj[q].x, g.L[0], code & 3);
+                const T dy = shifted_diff(xi.y, xi.y - g.L[1], xj[q].y, g.L[1], (code >> 2) & 3);
+                const T dz = shifted_diff(xi.z, xi.z - g.L[2], xj[q].z, g.L[2], code >> 4);
+                const T r2 = dx * dx + dy * dy + dz * dz;
+                if (r2 < rmax2) atomicAdd(&hist[rdf_bin(r2, inv_dr, inv_drf, nbins)], 1u);
             }
         }
     }
@@ -334,7 +383,7 @@ void Launch<T>::set_force(const DevSys<T>& s, const double* f, cudaStream_t st) 
 
 template <class T>
 void Launch<T>::reduce_obs(const DevSys<T>& s, double* out, cudaStream_t st) {
-    k_reduce_obs<T><<<s.R, 256, 0, st>>>(s, out);
+    k_reduce_obs<T><<<dim3(s.R, NPART), 256, 0, st>>>(s, out);
 }
 
 template <class T>
@@ -350,14 +399,14 @@ template <class T>
 void Launch<T>::rdf(const DevSys<T>& s, int cur, int rep, double rmax, int nbins,
                     unsigned long long* counts, cudaStream_t st) {
     k_rdf<T><<<4 * sm_count(), 256, sizeof(unsigned int) * nbins, st>>>(s, cur, rep, (T)(rmax * rmax),
-                                                                 nbins / rmax, nbins, counts);
+                                                                 nbins / rmax, (float)(nbins / rmax), nbins, counts);
 }
 
 template <class T>
 void Launch<T>::rdf_list(const DevSys<T>& s, int cur, int rep, double rmax, int nbins,
                          unsigned long long* counts, cudaStream_t st) {
     k_rdf_list<T><<<8 * sm_count(), 256, sizeof(unsigned int) * nbins, st>>>(s, cur, rep, (T)(rmax * rmax),
-                                                                      nbins / rmax, nbins, counts);
+                                                                      nbins / rmax, (float)(nbins / rmax), nbins, counts);
 }
 template void Launch<float>::rdf_list(const DevSys<float>&, int, int, double, int, unsigned long long*, cudaStream_t);
 template void Launch<double>::rdf_list(const DevSys<double>&, int, int, double, int, unsigned long long*, cudaStream_t);

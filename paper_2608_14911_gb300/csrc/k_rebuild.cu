@@ -193,7 +193,7 @@ template <class T, bool RANK>
 __device__ __forceinline__ int scan_count(const DevSys<T>& s, int k) {
     if (k >= s.ncells) return 0;
     const int c = RANK ? s.cell_by_rank[k] : k;
-    if (!RANK && s.now[s.cell_rep[c]]) return s.cell_cnt[c];
+    if (!RANK && s.now[s.R == 1 ? 0 : s.cell_rep[c]]) return s.cell_cnt[c];
     return s.cell_beg[c + 1] - s.cell_beg[c];
 }
 

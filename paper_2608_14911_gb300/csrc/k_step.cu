@@ -91,12 +91,6 @@ __global__ void __launch_bounds__(TILE) k_vsnap(DevSys<T> s) {
     }
 }
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // SH: launch shape (STEP_SHAPES) of the plain FP32 list path.  PPW: particles
 // per warp of the queue path (32, or 8 with four lanes per particle).
 template <class T, int MODE, bool ENERGY, bool FAST, bool DPD, bool LE, int SH = 0, int PPW = 32>
@@ -125,7 +119,8 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
     const V4<T>* __restrict__ P = s.pos[cur];
     V4<T>* __restrict__ Pn = s.pos[cur ^ 1];
     const IntParams<T>* __restrict__ ip = s.ip;
-    __shared__ double red[NPART][TILE / 32];
+    __shared__ double red[ENERGY ? NPART : 1][ENERGY ? TILE + 4 : 1];
+    static_assert(8 * NPART % 32 == 0 && 8 * NPART <= TILE, "whole warps reduce");
     __shared__ __align__(16) unsigned char queue_mem[QUEUE ? sizeof(PairQueue<T, DPD, PPW>) * (TILE / 32) : 16];
 
     for (int t = t0; t < s.ntiles; t += TPP > 1 ? s.ntiles : gridDim.x * TPB) {
@@ -359,18 +354,18 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
             acc[P_BOND_LEN] = 0.5 * blen;
             acc[P_BOND_CNT] = 0.5 * bcnt;
             acc[P_VIR_XZ] = 0.5 * (double)vxz;
-            const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+            // eight threads per quantity add 16 particles each, then each other's
+            // sums: a fifth of the FP64 additions of a tree over every warp
 #pragma unroll
-            for (int k = 0; k < NPART; ++k) {
-                const double r = warp_sum(acc[k]);
-                if (lane == 0) red[k][w] = r;
-            }
+            for (int k = 0; k < NPART; ++k) red[k][threadIdx.x] = acc[k];
             __syncthreads();
-            if (threadIdx.x < NPART) {
+            if (threadIdx.x < 8 * NPART) {
+                const int k = threadIdx.x >> 3, q = threadIdx.x & 7;
                 double sum = 0.0;
+                for (int j = 0; j < TILE / 8; ++j) sum += red[k][8 * j + q];
 #pragma unroll
-                for (int q = 0; q < TILE / 32; ++q) sum += red[threadIdx.x][q];
-                s.partials[(size_t)t * NPART + threadIdx.x] = sum;
+                for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                if (q == 0) s.partials[(size_t)t * NPART + k] = sum;
             }
             __syncthreads();
         }
