@@ -274,8 +274,9 @@ struct Ctrl {
                                // (inside an integrate call, after the first drift)
     unsigned int le_keep;      // the next rebuild keeps the stored Lees-Edwards build
                                // offsets (a checkpoint load), then clears this
+    int nact;                  // batches: tiles of the replicas being rebuilt
     // resident run kernel (k_run.cu)
-    unsigned int bar;          // arrivals at its grid barrier
+    unsigned int bar;          // arrivals at the grid barrier of a cooperative kernel
     long long target;          // last step of the run's segment
     long long stop;            // step after which a rebuild was requested or an error found
     int final_step;            // the segment's last step ends the integrate call

@@ -136,51 +136,88 @@ __device__ __forceinline__ void rank_particle(const DevSys<T>& s, const V4<T>* P
     if (s.cells_mode && s.dpd) s.cell_vel[b + rank] = s.vel[i];
 }
 
+// One block: the requests and, for batches, the list of the tiles to rebuild (in
+// a batch some replica asks at nearly every step, a tenth of them at a time).
 template <class T>
-__global__ void __launch_bounds__(256) k_latch(DevSys<T> s) {
+__global__ void __launch_bounds__(SCAN_THREADS) k_latch(DevSys<T> s) {
     if (s.ctrl->abort) return;
     latch_requests(s);
+    if (s.R == 1) return;
+    int carry = 0;
+    for (int r0 = 0; r0 < s.R; r0 += SCAN_THREADS) {
+        const int r = r0 + threadIdx.x;
+        const bool on = r < s.R && s.now[r] != 0;
+        const int a = on ? s.rep_tile_off[r] : 0, n = on ? s.rep_tile_off[r + 1] - a : 0;
+        int excl;
+        const int total = block_excl_scan(n, &excl);
+        for (int k = 0; k < n; ++k) s.act[carry + excl + k] = a + k;
+        carry += total;
+    }
+    if (threadIdx.x == 0) s.ctrl->nact = carry;
 }
 
 template <class T>
 __global__ void __launch_bounds__(TILE) k_bin(DevSys<T> s, int cur) {
-    // the first tile's record is requested together with the abort flag
-    Tile tl0 = {0, 0, 0, 0};
-    if ((int)blockIdx.x < s.ntiles) tl0 = ld_tile_early(s.tiles + blockIdx.x);
+    ActiveTiles<T> at(s);
     if (s.ctrl->abort) return;
     if (blockIdx.x == 0) clear_requests(s);
     V4<T>* P = s.pos[buffer_of(s, cur)];
-    for (int t = blockIdx.x; t < s.ntiles; t += gridDim.x) {
-        const Tile tl = t == (int)blockIdx.x ? tl0 : s.tiles[t];
-        if (!s.now[tl.rep] || (int)threadIdx.x >= tl.count) continue;
-        bin_particle(s, P, s.reps[tl.rep], tl.rep, tl.start + threadIdx.x);
-    }
+    Tile tl;
+    while (at.next(tl))
+        if ((int)threadIdx.x < tl.count) bin_particle(s, P, s.reps[tl.rep], tl.rep, tl.start + threadIdx.x);
 }
 
 template <class T>
 __global__ void __launch_bounds__(TILE) k_place(DevSys<T> s) {
-    // the first tile's record is requested together with the abort flag
-    Tile tl0 = {0, 0, 0, 0};
-    if ((int)blockIdx.x < s.ntiles) tl0 = ld_tile_early(s.tiles + blockIdx.x);
+    ActiveTiles<T> at(s);
     if (s.ctrl->abort) return;
-    for (int t = blockIdx.x; t < s.ntiles; t += gridDim.x) {
-        const Tile tl = t == (int)blockIdx.x ? tl0 : s.tiles[t];
-        if (!s.now[tl.rep] || (int)threadIdx.x >= tl.count) continue;
+    Tile tl;
+    while (at.next(tl)) {
         const int i = tl.start + threadIdx.x;
-        s.cell_slot[s.cell_beg[s.cellh[i]] + s.in_cell[i]] = i;
+        if ((int)threadIdx.x < tl.count) s.cell_slot[s.cell_beg[s.cellh[i]] + s.in_cell[i]] = i;
     }
 }
 
 template <class T>
 __global__ void __launch_bounds__(TILE) k_rank(DevSys<T> s, int cur) {
-    Tile tl0 = {0, 0, 0, 0};
-    if ((int)blockIdx.x < s.ntiles) tl0 = ld_tile_early(s.tiles + blockIdx.x);
+    ActiveTiles<T> at(s);
     if (s.ctrl->abort) return;
     const V4<T>* P = s.pos[buffer_of(s, cur)];
-    for (int t = blockIdx.x; t < s.ntiles; t += gridDim.x) {
-        const Tile tl = t == (int)blockIdx.x ? tl0 : s.tiles[t];
-        if (!s.now[tl.rep] || (int)threadIdx.x >= tl.count) continue;
-        rank_particle(s, P, tl.start + threadIdx.x);
+    Tile tl;
+    while (at.next(tl))
+        if ((int)threadIdx.x < tl.count) rank_particle(s, P, tl.start + threadIdx.x);
+}
+
+// Batches: one block per replica scans the cells of its replica alone, whose
+// entries start at its first slot (a scan over every replica's cells ran at
+// nearly every step of a batch for the tenth of them that had asked).
+template <class T>
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_replica(DevSys<T> s) {
+    if (s.ctrl->abort || !s.now[blockIdx.x]) return;
+    const RepGeom<T>& g = s.reps[blockIdx.x];
+    const int n = g.nc[0] * g.nc[1] * g.nc[2];
+    int* cnt = s.cell_cnt + g.cell_off;
+    int* beg = s.cell_beg + g.cell_off;
+    int carry = g.p_off;
+    for (int k0 = 0; k0 < n; k0 += SCAN_TILE) {
+        const int k = k0 + threadIdx.x * SCAN_ITEMS;
+        int v[SCAN_ITEMS], sum = 0, excl;
+#pragma unroll
+        for (int q = 0; q < SCAN_ITEMS; ++q) {
+            v[q] = k + q < n ? cnt[k + q] : 0;
+            sum += v[q];
+        }
+        const int total = block_excl_scan(sum, &excl);
+        int run = carry + excl;
+#pragma unroll
+        for (int q = 0; q < SCAN_ITEMS; ++q) {
+            if (k + q < n) {
+                beg[k + q] = run;
+                cnt[k + q] = 0;
+            }
+            run += v[q];
+        }
+        carry += total;
     }
 }
 
@@ -391,10 +428,10 @@ int binning_blocks() { return 4 * sm_count(); }
 // 9.42 / 9.18, of 200,000 29.2 / 29.5: beyond some 100,000 particles a kernel's own
 // blocks hide more latency than a barrier saves.
 template <class T>
-static bool binning_fused(const DevSys<T>& s) { return s.N < 100000; }
+static bool binning_fused(const DevSys<T>& s) { return s.N < 100000 && s.R == 1; }
 
 template <class T>
-int Launch<T>::binning_launches(const DevSys<T>& s) { return binning_fused(s) ? 1 : 7; }
+int Launch<T>::binning_launches(const DevSys<T>& s) { return binning_fused(s) ? 1 : s.R > 1 ? 5 : 7; }
 
 template <class T>
 int Launch<T>::rebuild(const DevSys<T>& s, int cur, bool resort, bool permute_force, cudaStream_t st) {
@@ -407,14 +444,19 @@ int Launch<T>::rebuild(const DevSys<T>& s, int cur, bool resort, bool permute_fo
         cudaLaunchCooperativeKernel((const void*)k_binning<T>, dim3(blocks), dim3(SCAN_THREADS), args, 0, st);
         launched = 1;
     } else {
-        k_latch<T><<<1, 256, 0, st>>>(s);
-        k_bin<T><<<gt, TILE, 0, st>>>(s, cur);
-        k_scan_reduce<T, false><<<s.nscan_blocks, SCAN_THREADS, 0, st>>>(s);
-        k_scan_top<T><<<1, SCAN_THREADS, 0, st>>>(s);
-        k_scan_down<T, false><<<s.nscan_blocks, SCAN_THREADS, 0, st>>>(s);
-        k_place<T><<<gt, TILE, 0, st>>>(s);
-        k_rank<T><<<gt, TILE, 0, st>>>(s, cur);
-        launched = 7;
+        const int ga = active_grid(s);
+        k_latch<T><<<1, SCAN_THREADS, 0, st>>>(s);
+        k_bin<T><<<ga, TILE, 0, st>>>(s, cur);
+        if (s.R > 1) {
+            k_scan_replica<T><<<s.R, SCAN_THREADS, 0, st>>>(s);
+        } else {
+            k_scan_reduce<T, false><<<s.nscan_blocks, SCAN_THREADS, 0, st>>>(s);
+            k_scan_top<T><<<1, SCAN_THREADS, 0, st>>>(s);
+            k_scan_down<T, false><<<s.nscan_blocks, SCAN_THREADS, 0, st>>>(s);
+        }
+        k_place<T><<<ga, TILE, 0, st>>>(s);
+        k_rank<T><<<ga, TILE, 0, st>>>(s, cur);
+        launched = binning_launches(s);
     }
     if (resort) {
         k_scan_reduce<T, true><<<s.nscan_blocks, SCAN_THREADS, 0, st>>>(s);

@@ -391,13 +391,10 @@ struct VerletSearch {
 template <class T, int W, bool EXCL, bool LE>
 __global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? 8 : 6) k_verlet(DevSys<T> s, int cur) {
     __shared__ int buf[TILE / 32][VB * 32];
-    // the first tile's record is requested together with the abort flag
-    Tile tl0 = {0, 0, 0, 0};
-    if ((int)blockIdx.x < s.ntiles) tl0 = ld_tile_early(s.tiles + blockIdx.x);
+    ActiveTiles<T> at(s);
     if (s.ctrl->abort) return;
-    for (int t = blockIdx.x; t < s.ntiles; t += gridDim.x) {
-        const Tile tl = t == (int)blockIdx.x ? tl0 : s.tiles[t];
-        if (!s.now[tl.rep]) continue;  // uniform over the block
+    Tile tl;
+    while (at.next(tl)) {  // (uniform over the block)
         VerletSearch<T, W, EXCL, LE, 1> v(s, s.reps[tl.rep]);
         v.EF = entries_f(s);
         v.P = sizeof(T) == 8 ? s.pos[buffer_of(s, cur)] : nullptr;  // (FP32 handles have no second test)
@@ -451,8 +448,8 @@ void Launch<T>::verlet(const DevSys<T>& s, int cur, cudaStream_t st) {
             if (s.le_on) k_verlet_team<T, W, E, true><<<s.ntiles * VTEAM, TILE, 0, st>>>(s, cur);               \
             else k_verlet_team<T, W, E, false><<<s.ntiles * VTEAM, TILE, 0, st>>>(s, cur);                      \
         } else {                                                                                           \
-            if (s.le_on) k_verlet<T, W, E, true><<<s.ntiles, TILE, 0, st>>>(s, cur);                            \
-            else k_verlet<T, W, E, false><<<s.ntiles, TILE, 0, st>>>(s, cur);                                   \
+            if (s.le_on) k_verlet<T, W, E, true><<<active_grid(s), TILE, 0, st>>>(s, cur);                            \
+            else k_verlet<T, W, E, false><<<active_grid(s), TILE, 0, st>>>(s, cur);                                   \
         }                                                                                                  \
     } while (0)
 #define ESPP_VERLET_W(E)                    \

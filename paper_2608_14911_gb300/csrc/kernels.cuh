@@ -102,6 +102,7 @@ template <class T> struct DevSys {
     int ntiles;
     const int* rep_tile_off;  // R + 1: first tile of each replica
     int* req;           // rebuild requested (per replica), set by the step kernel
+    int* act;           // batches: the tiles of the replicas being rebuilt (ctrl->nact of them)
     int* now;           // rebuild running (per replica), latched at the rebuild start
     Ctrl* ctrl;
     const IntParams<T>* ip;
@@ -238,6 +239,37 @@ __device__ __forceinline__ int cell_coord(T x, T cpl, int nc) {
     int c = (int)(x * cpl);
     c = c < 0 ? 0 : c;
     return c >= nc ? nc - 1 : c;
+}
+
+// The tiles of the replicas being rebuilt, taken by blocks in turn: every tile of a
+// single system, the listed ones of a batch.  The first tile's record is requested
+// at once, before the abort flag.
+template <class T>
+struct ActiveTiles {
+    const DevSys<T>& s;
+    int k, n;
+    bool first = true;
+    Tile tl0 = {0, 0, 0, 0};
+    __device__ __forceinline__ explicit ActiveTiles(const DevSys<T>& s_) : s(s_), k(blockIdx.x) {
+        if (s.R > 1) {
+            n = s.ctrl->nact;
+        } else {
+            if (k < s.ntiles) tl0 = ld_tile_early(s.tiles + k);
+            n = s.now[0] ? s.ntiles : 0;
+        }
+    }
+    __device__ __forceinline__ bool next(Tile& tl) {
+        if (!first) k += gridDim.x;
+        if (k >= n) return false;
+        tl = s.R > 1 ? s.tiles[s.act[k]] : first ? tl0 : s.tiles[k];
+        first = false;
+        return true;
+    }
+};
+// its grid: a batch rebuilds a part of its tiles at a time
+template <class T>
+int active_grid(const DevSys<T>& s) {
+    return s.R > 1 && s.ntiles > 16 * sm_count() ? 16 * sm_count() : s.ntiles;
 }
 
 // the cell entries in FP32, as the list search reads them

@@ -323,7 +323,7 @@ class System : public SystemBase {
         if ((rc = alloc(&bg, n, allocs)) || (rc = alloc(&sid, n, allocs)) ||
             (rc = alloc(&perm, n, allocs)) || (rc = alloc(&cellh, n, allocs)) ||
             (rc = alloc(&inc, n, allocs)) || (rc = alloc(&ncnt, n, allocs)) ||
-            (rc = alloc(&req, R, allocs)) || (rc = alloc(&now, R, allocs)) ||
+            (rc = alloc(&req, R, allocs)) || (rc = alloc(&now, R, allocs)) || (rc = alloc(&d.act, tiles_h.size(), allocs)) ||
             (rc = alloc(&tl, tiles_h.size(), allocs)) || (rc = alloc(&rto, R + 1, allocs)) ||
             (rc = alloc(&part, tiles_h.size() * NPART, allocs)) ||
             (rc = alloc(&d_geom, R, allocs)) || (rc = alloc(&d_ip, 1, allocs)) ||
