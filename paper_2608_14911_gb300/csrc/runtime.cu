@@ -176,6 +176,8 @@ class System : public SystemBase {
         if (tab_alloc) cudaFree(tab_alloc);
         if (d_hist) cudaFree(d_hist);
         for (void* p : allocs) cudaFree(p);
+        if (h_ctrl) cudaFreeHost(h_ctrl);
+        if (h_back) cudaFreeHost(h_back);
     }
 
     template <class P>
@@ -190,6 +192,19 @@ class System : public SystemBase {
         return ESPP_OK;
     }
 
+    // pinned room for results copied back (pageable copies wait one by one)
+    void* h_back = nullptr;
+    size_t h_back_bytes = 0;
+    int pinned_back(size_t bytes) {
+        if (bytes <= h_back_bytes) return ESPP_OK;
+        if (h_back) cudaFreeHost(h_back);
+        h_back = nullptr;
+        h_back_bytes = 0;
+        CK(cudaMallocHost(&h_back, bytes));
+        h_back_bytes = bytes;
+        return ESPP_OK;
+    }
+
     void clear_graphs() {
         for (auto& kv : graphs) {
             cudaGraphExecDestroy(kv.second.exec);
@@ -201,6 +216,7 @@ class System : public SystemBase {
 
     // ---------------------------------------------------------------- create
     int create(int Rr, const espp_replica_desc* descs, cudaStream_t stream) {
+        CK(cudaMallocHost(&h_ctrl, sizeof(Ctrl)));
         st = stream;
         R = Rr;
         for (int a = 0; a < MAX_TYPES; ++a) mass_h[a] = 1.0;
@@ -602,24 +618,27 @@ class System : public SystemBase {
         cur = 0;
         {
             // a new state clears any earlier error or freeze (the step number is kept)
-            Ctrl c = read_ctrl();
+            Ctrl c = ctrl_now();
             c.err = 0;
             c.abort = 0;
             c.any_req = 0;
             c.blocks_done = 0;
             c.need_cap = 0;
+            touch();
             CK(cudaMemcpyAsync(d_ctrl, &c, sizeof(Ctrl), cudaMemcpyHostToDevice, st));
         }
         Launch<T>::set_state(d, dx, dv, di, d_types, cur, st);
+        touch();
         Launch<T>::request_all(d, st);
         launches += 2;
         CK(cudaGetLastError());
-        CK(cudaStreamSynchronize(st));
         {
-            Ctrl c = read_ctrl();
+            Ctrl c = read_ctrl();  // waits: the caller's buffers are free again
+            if (!ctrl_known) return fail(ESPP_ERR_CUDA, cudaGetErrorString(cudaGetLastError()));
             if (c.err & ERRBIT_NONFINITE) {
                 // refuse the state: clear the flag, keep no half-set state
                 c.err = 0;
+                touch();
                 CK(cudaMemcpy(d_ctrl, &c, sizeof(Ctrl), cudaMemcpyHostToDevice));
                 state_set = false;
                 return fail(ESPP_ERR_ARG, "non-finite position or velocity");
@@ -653,18 +672,31 @@ class System : public SystemBase {
         return ESPP_OK;
     }
 
+    // The control block as it stands once the stream's work is done (waits for
+    // it), through a pinned copy; ctrl_now(): the same without the wait while
+    // nothing has been launched since (touch() is called before every launch
+    // or copy that may change it).
+    Ctrl* h_ctrl = nullptr;  // pinned
+    bool ctrl_known = false;
+    void touch() { ctrl_known = false; }
+    Ctrl ctrl_now() { return ctrl_known ? *h_ctrl : read_ctrl(); }
     Ctrl read_ctrl() {
         Ctrl c;
         memset(&c, 0, sizeof(c));
-        cudaMemcpyAsync(&c, d_ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st);
-        cudaStreamSynchronize(st);
+        ctrl_known = false;
+        if (cudaMemcpyAsync(h_ctrl, d_ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st) == cudaSuccess &&
+            cudaStreamSynchronize(st) == cudaSuccess) {
+            c = *h_ctrl;
+            ctrl_known = true;
+        }
         return c;
     }
 
     int set_step(int64_t s) override {
         // the simulated time stays; the step number it belongs to changes
-        Ctrl c = read_ctrl();
+        Ctrl c = ctrl_now();
         const double t = time_at(c.step);
+        touch();
         CK(cudaMemcpyAsync(&d_ctrl->step, &s, sizeof(long long), cudaMemcpyHostToDevice, st));
         CK(cudaStreamSynchronize(st));
         return set_clock(t, le_clk_h.dt, s);
@@ -679,15 +711,15 @@ class System : public SystemBase {
         // the kernels read the clock under Lees-Edwards only; switching it on
         // (or loading a sheared checkpoint) passes through here again
         if (!d.le_on) return ESPP_OK;
+        // (a few bytes from pageable memory: staged before the call returns)
         CK(cudaMemcpyAsync(d_le_clk, &le_clk_h, sizeof(LeClock), cudaMemcpyHostToDevice, st));
-        CK(cudaStreamSynchronize(st));
         return ESPP_OK;
     }
 
     int set_lees_edwards(int on, double shear, double time) override {
         if (!std::isfinite(shear) || !std::isfinite(time)) return fail(ESPP_ERR_ARG, "shear rate and time must be finite");
         if (on && d.mlp_on) return fail(ESPP_ERR_STATE, "Lees-Edwards is not available with the learned potential");
-        Ctrl c = read_ctrl();
+        Ctrl c = ctrl_now();
         d.le_on = on ? 1 : 0;
         d.le_shear = on ? shear : 0.0;
         int rcode = set_clock(time, le_clk_h.dt, c.step);
@@ -699,7 +731,7 @@ class System : public SystemBase {
     }
 
     int get_lees_edwards(int* on, double* shear, double* time) override {
-        Ctrl c = read_ctrl();
+        Ctrl c = ctrl_now();
         if (on) *on = d.le_on;
         if (shear) *shear = d.le_shear;
         if (time) *time = time_at(c.step);
@@ -900,6 +932,7 @@ class System : public SystemBase {
                     // a training frame needs its list, not a new storage order
                     rcode = rebuild_now(false, false);
                     if (rcode) return rcode;
+                    touch();
                     launches += Launch<T>::mlp_tc(d, cur, false, st);
                     launches += Launch<T>::train_grad(d, cur, Y + f * n3, t_err, t_loss_part, scale, t_partials,
                                                           t_blocks, t_grad, t_loss + ep, st);
@@ -946,6 +979,7 @@ class System : public SystemBase {
         clear_graphs();  // a kernel argument of the captured graphs
         rebuild_pending = true;
         if (state_set) {
+            touch();
             Launch<T>::request_all(d, st);
             launches++;
         }
@@ -1061,6 +1095,7 @@ class System : public SystemBase {
         if (!d.mlp_on || !d.nbr || (mlp_buf && mlp_buf_cap == d.cap)) return ESPP_OK;
         int rcode = alloc_mlp_buffers();
         if (rcode) return rcode;
+        touch();
         Launch<T>::request_all(d, st);
         launches++;
         rebuild_pending = true;
@@ -1138,6 +1173,7 @@ class System : public SystemBase {
         rcode = alloc_list(estimate_cap());
         if (rcode) return rcode;
         if (!state_set) return ESPP_OK;
+        touch();
         Launch<T>::request_all(d, st);
         launches++;
         return rebuild_now(f_valid);
@@ -1151,6 +1187,7 @@ class System : public SystemBase {
         NvtxRange nvtx_range("espp_rebuild");
         if (!cells_ready) return fail(ESPP_ERR_STATE, "call espp_build_neighbors first");
         for (int attempt = 0; attempt < 6; ++attempt) {
+            touch();
             launches += Launch<T>::rebuild(d, cur, resort, permute_force, st);
             CK(cudaGetLastError());
             Ctrl c = read_ctrl();
@@ -1180,7 +1217,9 @@ class System : public SystemBase {
         w.abort = 0;
         w.need_cap = 0;
         w.blocks_done = 0;
+        touch();
         CK(cudaMemcpyAsync(d_ctrl, &w, sizeof(Ctrl), cudaMemcpyHostToDevice, st));
+        touch();
         Launch<T>::request_all(d, st);
         launches++;
         CK(cudaStreamSynchronize(st));
@@ -1199,12 +1238,12 @@ class System : public SystemBase {
         if (rcode) return rcode;
         rcode = ensure_mlp_buffers();
         if (rcode) return rcode;
-        Ctrl c = read_ctrl();
+        Ctrl c = ctrl_now();
         if (c.abort) return status_from(c);
         if (rebuild_pending || c.any_req) {
             rcode = rebuild_now(f_valid);
             if (rcode) return rcode;
-            if (out) c = read_ctrl();
+            if (out) c = ctrl_now();
         }
         if (out) *out = c;
         return ESPP_OK;
@@ -1262,12 +1301,14 @@ class System : public SystemBase {
         double* target = f;
         if (f && where == ESPP_HOST) target = d_io_x;
         else if (f && where != ESPP_DEVICE) return fail(ESPP_ERR_ARG, "bad where");
+        touch();
         launches += Launch<T>::step(d, MODE_FORCES, false, cur, target, 0, 0, st);
         CK(cudaGetLastError());
         if (f && where == ESPP_HOST)
             CK(cudaMemcpyAsync(f, d_io_x, 3 * (size_t)N * sizeof(double), cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
-        return status_from(read_ctrl());
+        const Ctrl c = read_ctrl();
+        if (!ctrl_known) return fail(ESPP_ERR_CUDA, cudaGetErrorString(cudaGetLastError()));
+        return status_from(c);
     }
 
     // -------------------------------------------------------------- integrate
@@ -1488,9 +1529,11 @@ class System : public SystemBase {
         // the clock of this call: t(step0) carried over, this call's dt
         rcode = set_clock(time_at(step0), dt, step0);
         if (rcode) return rcode;
+        touch();
         if (!f_valid) {
             if (d.cells_mode && d.dpd) {
                 // the DPD pair term reads the cell-ordered velocities: bin again
+                touch();
                 Launch<T>::request_all(d, st);
                 launches += 1 + Launch<T>::rebuild(d, cur, false, false, st);
             }
@@ -1498,6 +1541,7 @@ class System : public SystemBase {
             f_valid = true;
         }
         const int c_start = cur;
+        touch();
         Launch<T>::prologue(d, cur, 0, st);
         launches++;
         CK(cudaGetLastError());
@@ -1512,6 +1556,7 @@ class System : public SystemBase {
                 // Hilbert resort (with a list rebuild) before every step that is
                 // a multiple of resort_every: a function of the step number only
                 if (resort_every > 0 && next % resort_every == 0) {
+                    touch();
                     Launch<T>::request_all(d, st);
                     launches += 1 + Launch<T>::rebuild(d, p, true, false, st);
                     host_rebuilds++;
@@ -1599,19 +1644,24 @@ class System : public SystemBase {
         if (rcode) return rcode;
         rcode = upload_int_params(ip_key[0] > 0 ? ip_key[0] : 1.0, std::max(ip_key[1], 0.0), std::max(ip_key[2], 0.0));
         if (rcode) return rcode;
+        touch();
         launches += Launch<T>::step(d, MODE_FORCES, true, cur, nullptr, 0, 0, st);
         Launch<T>::reduce_obs(d, d_obs, st);
         Launch<T>::rg2(d, cur, d_mol_members, d_mol_off, d_mol_rep, (int)mol_rep_h.size(), d_mol_rg2, st);
         launches += 2;
         CK(cudaGetLastError());
-        std::vector<double> part((size_t)R * NPART), rg(mol_rep_h.size());
-        CK(cudaMemcpyAsync(part.data(), d_obs, part.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
-        if (!rg.empty()) CK(cudaMemcpyAsync(rg.data(), d_mol_rg2, rg.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
+        const size_t npart = (size_t)R * NPART, nrg = mol_rep_h.size();
+        rcode = pinned_back((npart + nrg) * sizeof(double));
+        if (rcode) return rcode;
+        const double* part = static_cast<double*>(h_back);
+        const double* rg = part + npart;
+        CK(cudaMemcpyAsync(h_back, d_obs, npart * sizeof(double), cudaMemcpyDeviceToHost, st));
+        if (nrg) CK(cudaMemcpyAsync((double*)h_back + npart, d_mol_rg2, nrg * sizeof(double), cudaMemcpyDeviceToHost, st));
         Ctrl c = read_ctrl();
         CK(cudaGetLastError());
         std::vector<double> rgsum(R, 0.0);
         std::vector<int64_t> nmol(R, 0);
-        for (size_t m = 0; m < rg.size(); ++m) {
+        for (size_t m = 0; m < nrg; ++m) {
             rgsum[mol_rep_h[m]] += rg[m];
             nmol[mol_rep_h[m]]++;
         }
@@ -1669,8 +1719,10 @@ class System : public SystemBase {
         else Launch<T>::rdf(d, cur, rep, rmax, nbins, d_hist, st);
         launches++;
         CK(cudaGetLastError());
-        std::vector<unsigned long long> h(nbins);
-        CK(cudaMemcpyAsync(h.data(), d_hist, nbins * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+        const int rb = pinned_back(nbins * sizeof(unsigned long long));
+        if (rb) return rb;
+        const unsigned long long* h = static_cast<unsigned long long*>(h_back);
+        CK(cudaMemcpyAsync(h_back, d_hist, nbins * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
         for (int b = 0; b < nbins; ++b) counts[b] = (int64_t)h[b];
         return ESPP_OK;
@@ -1827,6 +1879,7 @@ class System : public SystemBase {
         rcode = set_clock(hd.le_time, hd.le_dt, hd.step);
         if (rcode) return rcode;
         Ctrl c = read_ctrl();
+        touch();
         c.step = hd.step;
         c.pos_ahead = 0;
         c.le_keep = 1;  // the list below is rebuilt with the saved build offsets
@@ -1839,12 +1892,14 @@ class System : public SystemBase {
         // the list of the saved run was built from the build positions: rebuild
         // it from them (buffer 1 holds a copy), without a resort
         // (list-free mode: bin the saved positions, which the last step binned)
+        touch();
         Launch<T>::request_all(d, st);
         launches += 1 + Launch<T>::rebuild(d, d.cells_mode ? 0 : 1, false, false, st);
         CK(cudaGetLastError());
         rebuild_pending = false;  // the loaded state is complete
         c = read_ctrl();
         if (c.err & ERRBIT_OVERFLOW) return fail(ESPP_ERR_LIST_OVERFLOW, "list capacity too small for the checkpoint");
+        touch();
         // restore the pending requests and the rebuild counter of the saved run
         CK(cudaMemcpy(d.req, req.data(), (size_t)R * sizeof(int), cudaMemcpyHostToDevice));
         int any = 0;
@@ -1859,11 +1914,11 @@ class System : public SystemBase {
     }
 
     // ------------------------------------------------------------ diagnostics
-    uint32_t error_word() override { return read_ctrl().err; }
+    uint32_t error_word() override { return ctrl_now().err; }
     int64_t num_particles() override { return N; }
     int32_t num_replicas() override { return R; }
-    int64_t num_rebuilds() override { return read_ctrl().n_rebuilds; }
-    int64_t step() override { return read_ctrl().step; }
+    int64_t num_rebuilds() override { return ctrl_now().n_rebuilds; }
+    int64_t step() override { return ctrl_now().step; }
     int32_t list_capacity() override { return d.cap; }
     int64_t kernel_launches() override { return launches; }
     int list_stats(int64_t* total, int32_t* maxc) override {
@@ -2111,6 +2166,7 @@ class System : public SystemBase {
         int rcode = upload_geometry();
         if (rcode) return rcode;
         const long long step = hs.step;
+        touch();
         CK(cudaMemcpyAsync(&d_ctrl->step, &step, sizeof(long long), cudaMemcpyHostToDevice, st));
         CK(cudaStreamSynchronize(st));
         if ((rcode = set_clock(hs.time, le_clk_h.dt, hs.step))) return rcode;
