@@ -492,8 +492,11 @@ __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_PER_SM) k_mlp_tc(DevSys<fl
             tc::tmem_ld8x2(lanes + c, lanes + 64 + c, y, dy);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const float2 bb = *reinterpret_cast<const float2*>(sh.b2h + c + 2 * j);
-                const float2 ww = *reinterpret_cast<const float2*>(sh.w3 + c + 2 * j);
+                // (16-byte loads of two units' pairs; the compiler shares them)
+                const float4 b4 = *reinterpret_cast<const float4*>(sh.b2h + c + 4 * (j >> 1));
+                const float4 w4 = *reinterpret_cast<const float4*>(sh.w3 + c + 4 * (j >> 1));
+                const float2 bb = j & 1 ? make_float2(b4.z, b4.w) : make_float2(b4.x, b4.y);
+                const float2 ww = j & 1 ? make_float2(w4.z, w4.w) : make_float2(w4.x, w4.y);
                 const f32x2 yv = f2add(f2(y[2 * j], y[2 * j + 1]), f2(bb.x, bb.y));
                 float y0, y1;
                 f2split(yv, y0, y1);
