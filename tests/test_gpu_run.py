@@ -63,3 +63,37 @@ def test_broken_bond_stops_the_run(prec):
     s.set_state(x, np.zeros_like(v), img)
     s.integrate(5, 0.001, 1.0, 0.1)
     s.close()
+
+
+def test_handles_on_streams_and_threads_run_together():
+    # resident kernels of several handles, each on its own stream and host
+    # thread: the same bits as one after the other
+    import threading
+    import torch
+    sizes = [(FP32, 20, 50), (FP32, 40, 100), (FP64, 20, 50), (FP32, 200, 128), (FP64, 100, 64), (FP32, 300, 128)]
+
+    def go(k, stream, out):
+        prec, chains, beads = sizes[k]
+        c = I.kg_lattice(chains, beads, density=0.85, seed=k)
+        s = espp.System(c.box, c.n, c.types, c.bonds, precision=prec, seed=k, stream=stream)
+        s.set_wca()
+        s.set_fene()
+        s.set_state(c.x, I.maxwell_velocities(c.n, 1.0, seed=k), c.img)
+        s.build_neighbors(WCA_RC, 0.4)
+        for n in (120, 1, 79):
+            s.integrate(n, 0.005, 1.0, 1.0)
+        out[k] = s.get_state()
+        s.close()
+
+    alone, together = {}, {}
+    for k in range(len(sizes)):
+        go(k, 0, alone)
+    streams = [torch.cuda.Stream() for _ in sizes]
+    threads = [threading.Thread(target=go, args=(k, streams[k].cuda_stream, together)) for k in range(len(sizes))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for k in range(len(sizes)):
+        for p, q in zip(alone[k], together[k]):
+            assert np.array_equal(p, q), k
