@@ -216,7 +216,6 @@ class System : public SystemBase {
 
     // ---------------------------------------------------------------- create
     int create(int Rr, const espp_replica_desc* descs, cudaStream_t stream) {
-        CK(cudaMallocHost(&h_ctrl, sizeof(Ctrl)));
         st = stream;
         R = Rr;
         for (int a = 0; a < MAX_TYPES; ++a) mass_h[a] = 1.0;
@@ -321,7 +320,8 @@ class System : public SystemBase {
             }
             rep_tile_off_h.push_back((int)tiles_h.size());
         }
-        // device buffers
+        // pinned mirror and device buffers, after every check of the arguments
+        CK(cudaMallocHost(&h_ctrl, sizeof(Ctrl)));
         int rc = ESPP_OK;
         const size_t n = (size_t)N;
         if ((rc = alloc(&d.pos[0], n + 1, allocs)) || (rc = alloc(&d.pos[1], n + 1, allocs)) ||
