@@ -464,7 +464,9 @@ int64_t espp_kernel_launches(espp_h h);
  * (sum of step-kernel ms, number of step-kernel launches timed, sum of
  * rebuild-node ms, number of steps timed); reset = 1 clears the sums.
  * Graphs with and without the timing events are cached side by side, so
- * switching does not rebuild them after the first use of each. */
+ * switching does not rebuild them after the first use of each.  Small handles
+ * that otherwise run many steps in one kernel take the step graphs while timing
+ * is enabled (the same results). */
 int espp_set_kernel_timing(espp_h h, int enable);
 int espp_kernel_timing(espp_h h, double* out, int reset);
 
@@ -492,7 +494,9 @@ int espp_set_resort_interval(espp_h h, int64_t steps);
  * ESPP_ERR_ARG unless 0 <= w <= 3, or for w = 3 in the list-free mode. */
 int espp_set_cell_subdivision(espp_h h, int32_t w);
 
-/* Steps captured per CUDA graph replay in espp_integrate (default 64).  0
+/* Steps captured per CUDA graph replay in espp_integrate (default 64; small
+ * handles of one Lennard-Jones / WCA type under Langevin run a whole segment in
+ * one graph whatever the value).  0
  * launches every kernel directly instead (no graphs; for profilers, which do
  * not see kernels inside conditional graphs). */
 int espp_set_graph_chunk(espp_h h, int32_t steps);
