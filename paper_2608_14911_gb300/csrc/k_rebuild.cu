@@ -298,7 +298,12 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_binning(DevSys<T> s, int cu
     constexpr int TB = SCAN_THREADS / TILE;
     Ctrl* c = s.ctrl;
     // no block changes these before every block has read them
-    if (c->abort || !c->any_req) return;
+    if (c->abort) return;
+    if (!c->any_req) {
+        // nothing is built: the kernels after this one read the latched flag
+        if (blockIdx.x == 0 && threadIdx.x == 0) s.now[0] = 0;
+        return;
+    }
     V4<T>* P = s.pos[buffer_of(s, cur)];
     const int lt = threadIdx.x % TILE, t0 = blockIdx.x * TB + threadIdx.x / TILE;
     unsigned int phase = 1;

@@ -49,6 +49,22 @@ def test_run_equals_single_launches(prec, chains, beads):
 
 
 @pytest.mark.parametrize("prec", [FP32, FP64])
+def test_direct_launches_keep_the_list_of_the_last_build(prec):
+    # the rebuild kernels launched at every step build only when a replica asked:
+    # the list held at the end is the last build's, whose pairs at the list radius
+    # are no longer where they were
+    lists = []
+    for chunk in (None, 0):
+        s = _melt(200, 100, prec, chunk)
+        s.integrate(57, 0.005, 1.0, 1.0)
+        lists.append((s.n_rebuilds, s.step) + tuple(s.get_neighbors()))
+        s.close()
+    a, b = lists
+    assert a[:2] == b[:2]
+    assert np.array_equal(a[2], b[2]) and np.array_equal(a[3], b[3])
+
+
+@pytest.mark.parametrize("prec", [FP32, FP64])
 def test_broken_bond_stops_the_run(prec):
     # a bond pulled past R0 by its beads' velocities, some steps into the run
     s = _melt(20, 50, prec)
