@@ -11,20 +11,22 @@ constexpr int GRID_WAIT = 1 << 21;  // polls before giving up (a second or so)
 // Barrier number `phase` (1, 2, ..) of this launch, called by every thread of
 // every block; false if the wait ran out (the error is recorded; the block is to
 // leave).  Writes before it are visible to plain loads after it.  after(): run by
-// thread 0 between the wait and the block's release.
+// thread 0 between the wait and the block's release.  fault: a barrier of the launch
+// whose wait runs out at once, whoever arrives (0: none; the tests' injection).
 template <class F>
-__device__ __forceinline__ bool grid_barrier(Ctrl* c, unsigned int phase, F&& after) {
+__device__ __forceinline__ bool grid_barrier(Ctrl* c, unsigned int phase, unsigned int fault, F&& after) {
     __shared__ int arrived;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        const unsigned int goal = gridDim.x * phase;
+        const unsigned int goal = gridDim.x * phase + (phase == fault ? 1u : 0u);
+        const int limit = phase == fault ? 64 : GRID_WAIT;
         atomicAdd(&c->bar, 1u);
         unsigned int seen = 0;
         int it = 0;
         do {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&c->bar) : "memory");
-        } while (seen < goal && ++it < GRID_WAIT);
+        } while (seen < goal && ++it < limit);
         __threadfence();
         after();
         arrived = seen >= goal;

@@ -297,8 +297,12 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_binning(DevSys<T> s, int cu
     static_assert(SCAN_THREADS % TILE == 0, "whole tiles per block");
     constexpr int TB = SCAN_THREADS / TILE;
     Ctrl* c = s.ctrl;
-    // no block changes these before every block has read them
-    if (c->abort) return;
+    // no block changes any_req before every block has read it; abort is set by a
+    // block whose wait ran out, and one that starts after that is counted as left
+    if (c->abort) {
+        grid_leave(c, [] {});
+        return;
+    }
     if (!c->any_req) {
         // nothing is built: the kernels after this one read the latched flag
         if (blockIdx.x == 0 && threadIdx.x == 0) s.now[0] = 0;
@@ -309,13 +313,13 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_binning(DevSys<T> s, int cu
     unsigned int phase = 1;
     bool ok = true;
     if (blockIdx.x == 0) latch_requests(s);
-    if (s.le_on) ok = grid_barrier(c, phase++, [] {});  // (bin reads the build's offset)
+    if (s.le_on) ok = grid_barrier(c, phase++, s.bin_fault, [] {});  // (bin reads the build's offset)
     if (ok)
         for (int t = t0; t < s.ntiles; t += gridDim.x * TB) {
             const Tile tl = s.tiles[t];
             if (s.req[tl.rep] && lt < tl.count) bin_particle(s, P, s.reps[tl.rep], tl.rep, tl.start + lt);
         }
-    ok = ok && grid_barrier(c, phase++, [] {});
+    ok = ok && grid_barrier(c, phase++, s.bin_fault, [] {});
     // the scan: every block one stretch of cells
     const int per = (s.ncells + gridDim.x - 1) / gridDim.x;
     const int c0 = min((int)blockIdx.x * per, s.ncells), c1 = min(c0 + per, s.ncells);
@@ -327,7 +331,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_binning(DevSys<T> s, int cu
         const int total = block_excl_scan(sum, &excl);
         if (threadIdx.x == 0) s.scan_part[blockIdx.x] = total;
     }
-    ok = ok && grid_barrier(c, phase++, [] {});
+    ok = ok && grid_barrier(c, phase++, s.bin_fault, [] {});
     if (ok) {
         int before = 0;
         for (int b = threadIdx.x; b < (int)blockIdx.x; b += SCAN_THREADS) before += s.scan_part[b];
@@ -343,14 +347,14 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_binning(DevSys<T> s, int cu
             carry += total;
         }
     }
-    ok = ok && grid_barrier(c, phase++, [] {});
+    ok = ok && grid_barrier(c, phase++, s.bin_fault, [] {});
     if (ok)
         for (int t = t0; t < s.ntiles; t += gridDim.x * TB) {
             const Tile tl = s.tiles[t];
             const int i = tl.start + lt;
             if (s.now[tl.rep] && lt < tl.count) s.cell_slot[s.cell_beg[s.cellh[i]] + s.in_cell[i]] = i;
         }
-    ok = ok && grid_barrier(c, phase++, [] {});
+    ok = ok && grid_barrier(c, phase++, s.bin_fault, [] {});
     if (ok)
         for (int t = t0; t < s.ntiles; t += gridDim.x * TB) {
             const Tile tl = s.tiles[t];

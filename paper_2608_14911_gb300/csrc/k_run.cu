@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(TILE, MINB) k_run(DevSys<T> s, unsigned long l
     const bool go = *(volatile unsigned int*)&c->abort == 0 && *(volatile unsigned int*)&c->any_req == 0 &&
                     step0 < target;
     unsigned int phase = 1;
-    bool ok = grid_barrier(c, phase++, [] {});
+    bool ok = grid_barrier(c, phase++, s.run_fault, [] {});
     long long step = step0;
     if (ok && go) {
         const int lt = TPP > 1 ? (int)(blockIdx.x % TPP) * (TILE / TPP) + (int)threadIdx.x / TPP : (int)threadIdx.x;
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(TILE, MINB) k_run(DevSys<T> s, unsigned long l
                 xi.y = __shfl_sync(0xffffffffu, xi.y, threadIdx.x & 28);
                 xi.z = __shfl_sync(0xffffffffu, xi.z, threadIdx.x & 28);
             }
-            ok = grid_barrier(c, phase++, [&] { stopped = *(volatile long long*)&c->stop; });
+            ok = grid_barrier(c, phase++, s.run_fault, [&] { stopped = *(volatile long long*)&c->stop; });
             if (!ok || step == target || stopped == step) break;
         }
         if (lead) s.vel[i] = v;

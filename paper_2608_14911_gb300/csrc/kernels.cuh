@@ -102,6 +102,8 @@ template <class T> struct DevSys {
     int ntiles;
     const int* rep_tile_off;  // R + 1: first tile of each replica
     int* req;           // rebuild requested (per replica), set by the step kernel
+    // fault injection (tests): the barrier of k_binning, k_run whose wait runs out
+    unsigned int bin_fault, run_fault;
     int* act;           // batches: the tiles of the replicas being rebuilt (ctrl->nact of them)
     int* now;           // rebuild running (per replica), latched at the rebuild start
     Ctrl* ctrl;

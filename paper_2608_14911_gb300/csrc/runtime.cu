@@ -370,6 +370,13 @@ class System : public SystemBase {
         }
         // host-side fault injection for tests: the tensor-core kernel's wait runs out
         if (const char* f = getenv("ESPP_FAULT_TC_TIMEOUT")) d.tc_fault = atoi(f) > 0 ? 1 : 0;
+        // ... the k-th grid barrier of the binning (k > 0) or run (-k) kernel's
+        // does, until a new state clears the error
+        if (const char* f = getenv("ESPP_FAULT_GRID_TIMEOUT")) {
+            const int k = atoi(f);
+            d.bin_fault = k > 0 ? k : 0;
+            d.run_fault = k < 0 ? -k : 0;
+        }
         d.bond_gid = bg;
         d.slot_of_id = sid;
         d.perm = perm;
@@ -596,6 +603,26 @@ class System : public SystemBase {
     bool mass_dirty = true;
 
     // ------------------------------------------------------------------ state
+    // Clears errors and requests in c.  A wait that ran out left the kernel's later
+    // phases undone: the counts of its binning, which every build finds at zero,
+    // are set back with it.
+    int clear_error(Ctrl& c) {
+        if (c.err & ERRBIT_TIMEOUT) {
+            if (cells_ready) CK(cudaMemsetAsync(d.cell_cnt, 0, (size_t)d.ncells * sizeof(int), st));
+            if (d.bin_fault || d.run_fault) {
+                d.bin_fault = d.run_fault = 0;
+                clear_graphs();  // kernel arguments of the captured graphs
+            }
+        }
+        c.err = 0;
+        c.abort = 0;
+        c.any_req = 0;
+        c.blocks_done = 0;
+        c.bar = 0;
+        c.need_cap = 0;
+        return ESPP_OK;
+    }
+
     int set_state(const double* x, const double* v, const int32_t* img, int where) override {
         if (!x) return fail(ESPP_ERR_ARG, "positions are required");
         const size_t n3 = 3 * (size_t)N;
@@ -619,11 +646,8 @@ class System : public SystemBase {
         {
             // a new state clears any earlier error or freeze (the step number is kept)
             Ctrl c = ctrl_now();
-            c.err = 0;
-            c.abort = 0;
-            c.any_req = 0;
-            c.blocks_done = 0;
-            c.need_cap = 0;
+            const int rc = clear_error(c);
+            if (rc) return rc;
             touch();
             CK(cudaMemcpyAsync(d_ctrl, &c, sizeof(Ctrl), cudaMemcpyHostToDevice, st));
         }
@@ -1192,6 +1216,7 @@ class System : public SystemBase {
             CK(cudaGetLastError());
             Ctrl c = read_ctrl();
             CK(cudaGetLastError());
+            if (c.err & ERRBIT_TIMEOUT) return status_from(c);  // the list is not built
             if (!(c.err & ERRBIT_OVERFLOW)) {
                 rebuild_pending = false;
                 return ESPP_OK;
@@ -1217,6 +1242,7 @@ class System : public SystemBase {
         w.abort = 0;
         w.need_cap = 0;
         w.blocks_done = 0;
+        w.bar = 0;
         touch();
         CK(cudaMemcpyAsync(d_ctrl, &w, sizeof(Ctrl), cudaMemcpyHostToDevice, st));
         touch();
@@ -1883,12 +1909,8 @@ class System : public SystemBase {
         c.step = hd.step;
         c.pos_ahead = 0;
         c.le_keep = 1;  // the list below is rebuilt with the saved build offsets
-        c.err = 0;
-        c.abort = 0;
-        c.any_req = 0;
-        c.blocks_done = 0;
-        c.need_cap = 0;
-        CK(cudaMemcpy(d_ctrl, &c, sizeof(Ctrl), cudaMemcpyHostToDevice));
+        if ((rcode = clear_error(c))) return rcode;
+        CK(cudaMemcpyAsync(d_ctrl, &c, sizeof(Ctrl), cudaMemcpyHostToDevice, st));
         // the list of the saved run was built from the build positions: rebuild
         // it from them (buffer 1 holds a copy), without a resort
         // (list-free mode: bin the saved positions, which the last step binned)
@@ -1899,6 +1921,7 @@ class System : public SystemBase {
         rebuild_pending = false;  // the loaded state is complete
         c = read_ctrl();
         if (c.err & ERRBIT_OVERFLOW) return fail(ESPP_ERR_LIST_OVERFLOW, "list capacity too small for the checkpoint");
+        if (c.err & ERRBIT_TIMEOUT) return status_from(c);
         touch();
         // restore the pending requests and the rebuild counter of the saved run
         CK(cudaMemcpy(d.req, req.data(), (size_t)R * sizeof(int), cudaMemcpyHostToDevice));

@@ -113,3 +113,58 @@ def test_handles_on_streams_and_threads_run_together():
     for k in range(len(sizes)):
         for p, q in zip(alone[k], together[k]):
             assert np.array_equal(p, q), k
+
+
+@pytest.mark.parametrize("prec", [FP32, FP64])
+@pytest.mark.parametrize("barrier,shear", [(1, False), (2, False), (4, False), (1, True), (5, True), (-1, False),
+                                           (-4, False)])
+def test_grid_barrier_timeout_is_reported_and_cleared(prec, barrier, shear, monkeypatch, tmp_path):
+    # host-side fault injection: one grid barrier's bounded wait of the binning
+    # (barrier > 0) or run kernel (< 0) runs out.  The call reports it, and a new
+    # state (or a loaded checkpoint) leaves nothing of it behind: the lists and
+    # trajectories are those of a handle that never failed
+    c = I.kg_lattice(40, 100, density=0.85, seed=4)
+    v = I.maxwell_velocities(c.n, 1.0, seed=4)
+
+    def handle():
+        s = espp.System(c.box, c.n, c.types, c.bonds, precision=prec, seed=4)
+        s.set_wca()
+        s.set_fene()
+        if shear:
+            s.set_lees_edwards(True, 0.1, 0.5)
+        s.set_state(c.x, v, c.img)
+        return s
+
+    good = handle()
+    good.build_neighbors(WCA_RC, 0.4)
+    path = str(tmp_path / "start")
+    good.checkpoint_save(path)
+    lists = good.get_neighbors()
+    good.integrate(40, 0.005, 1.0, 1.0)
+    for how in ("state", "checkpoint"):
+        monkeypatch.setenv("ESPP_FAULT_GRID_TIMEOUT", str(barrier))
+        s = handle()
+        monkeypatch.delenv("ESPP_FAULT_GRID_TIMEOUT")
+        with pytest.raises(espp.EsppError) as e:
+            s.build_neighbors(WCA_RC, 0.4)
+            s.integrate(40, 0.005, 1.0, 1.0)
+        assert e.value.code == espp.ESPP_ERR_TIMEOUT
+        with pytest.raises(espp.EsppError) as e:
+            s.compute_forces()
+        assert e.value.code == espp.ESPP_ERR_TIMEOUT
+        if how == "state":
+            s.set_step(0)
+            if shear:
+                s.set_lees_edwards(True, 0.1, 0.5)
+            s.set_state(c.x, v, c.img)
+            s.build_neighbors(WCA_RC, 0.4)
+        else:
+            s.checkpoint_load(path)
+        for a, b in zip(lists, s.get_neighbors()):
+            assert np.array_equal(a, b)
+        s.integrate(40, 0.005, 1.0, 1.0)
+        assert s.error_word == 0 and s.step == 40
+        for a, b in zip(good.get_state(), s.get_state()):
+            assert np.array_equal(a, b)
+        s.close()
+    good.close()
