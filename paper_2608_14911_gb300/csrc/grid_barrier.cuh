@@ -3,6 +3,7 @@
 // leave the kernel resets the count.
 #pragma once
 #include "common.cuh"
+#include "grid_count.h"
 
 namespace espp {
 
@@ -19,18 +20,19 @@ __device__ __forceinline__ bool grid_barrier(Ctrl* c, unsigned int phase, unsign
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        const unsigned int goal = gridDim.x * phase + (phase == fault ? 1u : 0u);
-        const int limit = phase == fault ? 64 : GRID_WAIT;
+        const bool never = fault != 0 && phase == fault;
+        const unsigned int goal = barrier_goal(gridDim.x, phase) + (never ? 1u : 0u);
+        const int limit = never ? 64 : GRID_WAIT;
         atomicAdd(&c->bar, 1u);
         unsigned int seen = 0;
         int it = 0;
         do {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&c->bar) : "memory");
-        } while (seen < goal && ++it < limit);
+        } while (!barrier_reached(seen, goal) && ++it < limit);
         __threadfence();
         after();
-        arrived = seen >= goal;
-        if (seen < goal) {
+        arrived = barrier_reached(seen, goal);
+        if (!arrived) {
             atomicOr(&c->err, ERRBIT_TIMEOUT);
             c->abort = 1;
         }

@@ -153,3 +153,40 @@ def test_noalloc_binding_refuses_wrong_tensors_before_the_call(lib):
                                      torch.zeros(8, dtype=torch.int64))
     with pytest.raises(ValueError):
         espp.espp_rdf_counts_noalloc(np.zeros((4, 3)), _BOX, 2.0, np.zeros(8, dtype=np.int64))
+
+
+GRID_COUNT = r"""
+#include "grid_count.h"
+#include <cstdio>
+int main() {
+    const unsigned int sizes[] = {1, 3, 606, 608, 912};
+    for (unsigned int blocks : sizes) {
+        const unsigned int wrap = (unsigned int)(0x100000000ull / blocks);
+        for (int k = -2; k <= 4; ++k) {
+            const unsigned int phase = k < 0 ? 3u + k : wrap - 2u + k;  // the first ones, those around 2^32 arrivals
+            const unsigned int goal = espp::barrier_goal(blocks, phase);
+            unsigned int count = blocks * (phase - 1u);  // everyone has passed the barrier before
+            for (unsigned int b = 0; b < 2 * blocks; ++b, ++count)
+                if (espp::barrier_reached(count, goal) != (b >= blocks)) {
+                    printf("blocks %u phase %u arrivals %u\n", blocks, phase, b);
+                    return 1;
+                }
+        }
+    }
+    return 0;
+}
+"""
+
+
+def test_grid_barrier_opens_once_every_block_has_arrived(tmp_path):
+    # the barrier's count passes 2^32 in a long run without a rebuild
+    import shutil
+    import subprocess
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if cxx is None:
+        pytest.skip("no C++ compiler")
+    src, exe = tmp_path / "count.cpp", str(tmp_path / "count")
+    src.write_text(GRID_COUNT)
+    subprocess.run([cxx, "-std=c++17", "-O1", "-Wall", "-Werror", "-I", pbuild.CSRC, str(src), "-o", exe], check=True)
+    out = subprocess.run([exe], capture_output=True, text=True, timeout=60)
+    assert out.returncode == 0, out.stdout
