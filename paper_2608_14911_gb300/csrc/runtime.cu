@@ -617,6 +617,7 @@ class System : public SystemBase {
         c.err = 0;
         c.abort = 0;
         c.any_req = 0;
+        c.pos_ahead = 0;  // the new positions are those of c.step
         c.blocks_done = 0;
         c.bar = 0;
         c.need_cap = 0;
@@ -1907,7 +1908,6 @@ class System : public SystemBase {
         Ctrl c = read_ctrl();
         touch();
         c.step = hd.step;
-        c.pos_ahead = 0;
         c.le_keep = 1;  // the list below is rebuilt with the saved build offsets
         if ((rcode = clear_error(c))) return rcode;
         CK(cudaMemcpyAsync(d_ctrl, &c, sizeof(Ctrl), cudaMemcpyHostToDevice, st));

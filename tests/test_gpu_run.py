@@ -168,3 +168,35 @@ def test_grid_barrier_timeout_is_reported_and_cleared(prec, barrier, shear, monk
             assert np.array_equal(a, b)
         s.close()
     good.close()
+
+
+def test_new_state_after_an_error_under_shear():
+    # a run frozen by a broken bond had the positions of the step after; a new
+    # state's belong to the step itself, Lees-Edwards offset included
+    c = I.kg_lattice(40, 100, density=0.85, seed=4)
+    v = I.maxwell_velocities(c.n, 1.0, seed=4)
+    fast = v.copy()
+    fast[0], fast[1] = (-60.0, 0.0, 0.0), (60.0, 0.0, 0.0)
+    out = []
+    for fails in (False, True):
+        s = espp.System(c.box, c.n, c.types, c.bonds, precision=FP64, seed=4)
+        s.set_wca()
+        s.set_fene()
+        s.set_lees_edwards(True, 0.4, 0.5)
+        s.set_state(c.x, fast if fails else v, c.img)
+        s.build_neighbors(WCA_RC, 0.4)
+        if fails:
+            with pytest.raises(espp.EsppError):
+                s.integrate(100, 0.005, 0.0, 0.0)
+        else:
+            s.integrate(1, 0.005, 0.0, 0.0)
+        s.set_step(0)
+        s.set_lees_edwards(True, 0.4, 0.5)
+        s.set_state(c.x, v, c.img)
+        obs = s.observables()
+        del obs["n_rebuilds"]  # (of the handle's life)
+        out.append((s.get_neighbors(), obs, s.compute_forces()))
+        s.close()
+    (la, oa, fa), (lb, ob, fb) = out
+    assert np.array_equal(la[0], lb[0]) and np.array_equal(la[1], lb[1])
+    assert oa == ob and np.array_equal(fa, fb)
