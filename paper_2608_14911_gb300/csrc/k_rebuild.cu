@@ -432,6 +432,15 @@ static inline int grid_for(int n, int block) { return (n + block - 1) / block; }
 // Blocks of the fused binning: four an SM are resident at once (its launch bounds).
 int binning_blocks() { return 4 * sm_count(); }
 
+// The fused binning has a block for every SCAN_THREADS particles, and for every
+// BIN_CELLS cells: in a dilute system the scan is most of its work.  us per step,
+// blocks by particles alone / by both / kernels of their own (list; cells): gas of
+// 1,000 in 287,000 cells 34.8 / 14.5 / 14.8, 577 / 32.0 / 41.3 (in 730,000); of 20,000
+// 17.7 / 16.7 / 16.6, 62.6 / 41.6 / 47.7; of 90,000 in 2.3 million 20.6 / 19.8 / 20.8, 93
+// / 73.5 / 110.  BIN_CELLS of 256 and 4096 instead of 1024: 5,000 in 62,000 (cells)
+// 32.0 and 39.2 against 30.4, dense systems the same.
+constexpr int BIN_CELLS = 4 * SCAN_THREADS;
+
 // us per step, kernels of their own / fused: DPD fluid in cells (binned every
 // step) 24,000 63.4 / 60.1, 98,304 91.2 / 90.0, 192,000 135 / 139; KG melt of 5,000
 // 9.42 / 9.18, of 200,000 29.2 / 29.5: beyond some 100,000 particles a kernel's own
@@ -449,7 +458,7 @@ int Launch<T>::rebuild(const DevSys<T>& s, int cur, bool resort, bool permute_fo
     if (binning_fused(s)) {
         DevSys<T> a = s;
         void* args[] = {&a, &cur};
-        const int blocks = std::min((gt + SCAN_THREADS / TILE - 1) / (SCAN_THREADS / TILE), binning_blocks());
+        const int blocks = std::min(std::max(grid_for(s.N, SCAN_THREADS), grid_for(s.ncells, BIN_CELLS)), binning_blocks());
         cudaLaunchCooperativeKernel((const void*)k_binning<T>, dim3(blocks), dim3(SCAN_THREADS), args, 0, st);
         launched = 1;
     } else {

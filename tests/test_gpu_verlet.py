@@ -10,6 +10,8 @@ import pytest
 import oracle as O
 from paper_2608_14911_gb300 import espp, inputs as I
 
+from _systems import rel_rms
+
 pytestmark = pytest.mark.gpu
 FP32, FP64 = espp.ESPP_FP32, espp.ESPP_FP64
 RL = 1.5
@@ -92,3 +94,30 @@ def test_both_forms_build_the_same_lists(prec, n):
         assert np.array_equal(f, fb[sl])
         for a, p in zip(q, st):
             assert np.array_equal(a, p[sl])
+
+
+@pytest.mark.parametrize("prec,tol,band", [(FP32, 1e-5, 1e-6), (FP64, 1e-12, 0.0)])
+@pytest.mark.parametrize("n,box", [
+    (1, (30.0, 4.6, 45.0)),           # 1800 cells, one particle
+    (100, (9.5, 24.2, 16.6)),         # 1056 cells: just past a block's share
+    (1000, (151.0, 64.0, 47.0)),      # 130,000 cells
+    (3000, (700.0, 31.0, 5.0)),       # a long flat box
+    (1500, (160.0, 151.0, 155.0)),    # 1.1 million cells: past the shares of all resident blocks
+])
+def test_dilute_boxes(prec, tol, band, n, box):
+    # many more cells than particles, whose scan has blocks of its own
+    c = _gas(n, box, 7 + n, min(n, 60))
+    s = _handle(c, prec, 1)
+    row, cols = s.get_neighbors()
+    s.set_force_method(espp.ESPP_FORCES_CELLS)
+    f = s.compute_forces()
+    s.close()
+    orow, ocols = O.neighbors(c.box, c.x, RL, method="brute")
+    for i in range(c.n):
+        for j in set(cols[row[i]:row[i + 1]].tolist()) ^ set(ocols[orow[i]:orow[i + 1]].tolist()):
+            d = c.x[i] - c.x[j]
+            d -= c.box * np.round(d / c.box)
+            assert abs(np.linalg.norm(d) - RL) <= band, (i, j)
+    m = O.Model(1, {(0, 0): ("lj_capped", 1.0, 1.0, 1.1, True, 0.8)}, None)
+    fo, _ = O.forces(m, c.box, c.x, c.types, c.bonds)
+    assert rel_rms(f, fo) <= tol
