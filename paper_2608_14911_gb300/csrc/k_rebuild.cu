@@ -150,7 +150,18 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_latch(DevSys<T> s) {
         const int a = on ? s.rep_tile_off[r] : 0, n = on ? s.rep_tile_off[r + 1] - a : 0;
         int excl;
         const int total = block_excl_scan(n, &excl);
-        for (int k = 0; k < n; ++k) s.act[carry + excl + k] = a + k;
+        // a thread writes its replica's tiles; a warp with a large replica among its
+        // 32 writes them together, one replica after the other
+        if (__any_sync(0xffffffffu, n > 128)) {
+            for (unsigned int left = __ballot_sync(0xffffffffu, n > 0); left; left &= left - 1) {
+                const int q = __ffs(left) - 1;
+                const int to = carry + __shfl_sync(0xffffffffu, excl, q), from = __shfl_sync(0xffffffffu, a, q),
+                          m = __shfl_sync(0xffffffffu, n, q);
+                for (int k = threadIdx.x & 31; k < m; k += 32) s.act[to + k] = from + k;
+            }
+        } else {
+            for (int k = 0; k < n; ++k) s.act[carry + excl + k] = a + k;
+        }
         carry += total;
     }
     if (threadIdx.x == 0) s.ctrl->nact = carry;
@@ -188,9 +199,9 @@ __global__ void __launch_bounds__(TILE) k_rank(DevSys<T> s, int cur) {
         if ((int)threadIdx.x < tl.count) rank_particle(s, P, tl.start + threadIdx.x);
 }
 
-// Batches: one block per replica scans the cells of its replica alone, whose
-// entries start at its first slot (a scan over every replica's cells ran at
-// nearly every step of a batch for the tenth of them that had asked).
+// Batches of small replicas: one block per replica scans the cells of its replica
+// alone, whose entries start at its first slot (a scan over every replica's cells
+// ran at nearly every step of a batch for the tenth of them that had asked).
 template <class T>
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_replica(DevSys<T> s) {
     if (s.ctrl->abort || !s.now[blockIdx.x]) return;
@@ -224,14 +235,22 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_replica(DevSys<T> s) {
 // ---- exclusive scan of the cell counts (three phases, no inter-block waits) --
 // RANK = false: cells in index order -> cell_beg (every rebuild);
 // RANK = true: cells in Hilbert-rank order -> rank_start, by cell (resort only).
-// The counts of this build are in cell_cnt, which is zero between builds; a cell
-// of a replica that is not rebuilt keeps the count its entries have.
+// The counts of this build are in cell_cnt, which is zero between builds.  A
+// replica that is not rebuilt counts all its particles in its last cell: what comes
+// after starts where it did, and its own cells are neither read nor written.
 template <class T, bool RANK>
-__device__ __forceinline__ int scan_count(const DevSys<T>& s, int k) {
+__device__ __forceinline__ int scan_count(const DevSys<T>& s, int k, bool& build) {
+    build = false;
     if (k >= s.ncells) return 0;
-    const int c = RANK ? s.cell_by_rank[k] : k;
-    if (!RANK && s.now[s.R == 1 ? 0 : s.cell_rep[c]]) return s.cell_cnt[c];
-    return s.cell_beg[c + 1] - s.cell_beg[c];
+    if (RANK) {
+        const int c = s.cell_by_rank[k];
+        return s.cell_beg[c + 1] - s.cell_beg[c];
+    }
+    const int r = s.R == 1 ? 0 : s.cell_rep[k];
+    build = s.now[r] != 0;
+    if (build) return s.cell_cnt[k];
+    if (s.R == 1 || (k + 1 < s.ncells && s.cell_rep[k + 1] == r)) return 0;
+    return (r + 1 < s.R ? s.reps[r + 1].p_off : s.N) - s.reps[r].p_off;
 }
 
 template <class T, bool RANK>
@@ -239,8 +258,9 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_reduce(DevSys<T> s) {
     if (s.ctrl->abort) return;
     const int base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
     int sum = 0;
+    bool build;
 #pragma unroll
-    for (int k = 0; k < SCAN_ITEMS; ++k) sum += scan_count<T, RANK>(s, base + k);
+    for (int k = 0; k < SCAN_ITEMS; ++k) sum += scan_count<T, RANK>(s, base + k, build);
     int excl;
     const int total = block_excl_scan(sum, &excl);
     if (threadIdx.x == 0) s.scan_part[blockIdx.x] = total;
@@ -265,10 +285,11 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_down(DevSys<T> s) {
     if (s.ctrl->abort) return;
     const int base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
     int v[SCAN_ITEMS];
+    bool build[SCAN_ITEMS];
     int sum = 0;
 #pragma unroll
     for (int k = 0; k < SCAN_ITEMS; ++k) {
-        v[k] = scan_count<T, RANK>(s, base + k);
+        v[k] = scan_count<T, RANK>(s, base + k, build[k]);
         sum += v[k];
     }
     int excl;
@@ -279,7 +300,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_down(DevSys<T> s) {
         if (base + k < s.ncells) {
             if (RANK) {
                 s.rank_start[s.cell_by_rank[base + k]] = run;
-            } else {
+            } else if (build[k]) {
                 s.cell_beg[base + k] = run;
                 s.cell_cnt[base + k] = 0;
             }
@@ -327,7 +348,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_binning(DevSys<T> s, int cu
     if (ok) {
         if (blockIdx.x == 0) clear_requests(s);
         int sum = 0;
-        for (int k = c0 + threadIdx.x; k < c1; k += SCAN_THREADS) sum += scan_count<T, false>(s, k);
+        for (int k = c0 + threadIdx.x; k < c1; k += SCAN_THREADS) sum += s.cell_cnt[k];
         const int total = block_excl_scan(sum, &excl);
         if (threadIdx.x == 0) s.scan_part[blockIdx.x] = total;
     }
@@ -338,7 +359,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_binning(DevSys<T> s, int cu
         int carry = block_excl_scan(before, &excl);
         for (int k0 = c0; k0 < c1; k0 += SCAN_THREADS) {
             const int k = k0 + threadIdx.x;
-            const int v = k < c1 ? scan_count<T, false>(s, k) : 0;
+            const int v = k < c1 ? s.cell_cnt[k] : 0;
             const int total = block_excl_scan(v, &excl);
             if (k < c1) {
                 s.cell_beg[k] = carry + excl;
@@ -448,8 +469,20 @@ constexpr int BIN_CELLS = 4 * SCAN_THREADS;
 template <class T>
 static bool binning_fused(const DevSys<T>& s) { return s.N < 100000 && s.R == 1; }
 
+// A batch's cells: a block per replica, or all cells by the three phases where a
+// cell's replica has many of them (the mean over cells, so that one large replica
+// does not decide for hundreds of small ones).  us per step, by replica / three
+// phases, KG melts on whole cells: 64 x 10,000 beads (2,700 cells) 94.4 / 97.3, 64 x
+// 20,000 (5,800) 137.7 / 139.8, 64 uneven ones (10,600) 171 / 161, 64 x 50,000
+// (15,600) 275 / 265, 4 x 100,000 (32,000) 65 / 51, 2 x 1,000,000 276 / 159.  The line lies
+// above where the times cross: two more kernels in every captured step make a new
+// handle's first call longer (the uneven batch's 10.0 -> 11.3 ms).
+constexpr int SCAN_REP_CELLS = 16384;
 template <class T>
-int Launch<T>::binning_launches(const DevSys<T>& s) { return binning_fused(s) ? 1 : s.R > 1 ? 5 : 7; }
+static bool scan_by_replica(const DevSys<T>& s) { return s.R > 1 && s.rep_cells <= SCAN_REP_CELLS; }
+
+template <class T>
+int Launch<T>::binning_launches(const DevSys<T>& s) { return binning_fused(s) ? 1 : scan_by_replica(s) ? 5 : 7; }
 
 template <class T>
 int Launch<T>::rebuild(const DevSys<T>& s, int cur, bool resort, bool permute_force, cudaStream_t st) {
@@ -465,7 +498,7 @@ int Launch<T>::rebuild(const DevSys<T>& s, int cur, bool resort, bool permute_fo
         const int ga = active_grid(s);
         k_latch<T><<<1, SCAN_THREADS, 0, st>>>(s);
         k_bin<T><<<ga, TILE, 0, st>>>(s, cur);
-        if (s.R > 1) {
+        if (scan_by_replica(s)) {
             k_scan_replica<T><<<s.R, SCAN_THREADS, 0, st>>>(s);
         } else {
             k_scan_reduce<T, false><<<s.nscan_blocks, SCAN_THREADS, 0, st>>>(s);

@@ -93,6 +93,7 @@ template <class T> struct DevSys {
     const int* cell_by_rank;  // global Hilbert rank -> cell index
     const int* cell_rep;
     int ncells;
+    int rep_cells;      // cells of a replica, averaged over all cells
     int* scan_part;
     int nscan_blocks;
     // replicas and tiles

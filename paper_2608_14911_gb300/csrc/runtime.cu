@@ -1154,10 +1154,12 @@ class System : public SystemBase {
         clear_graphs();
         std::vector<int> rep_of, by_rank;
         int coff = 0;
+        double nc2 = 0;
         for (int r = 0; r < R; ++r) {
             const int w = cell_sub;
             const int nx = cell_count(r, 0, w), ny = cell_count(r, 1, w), nz = cell_count(r, 2, w);
             const int nc = nx * ny * nz;
+            nc2 += (double)nc * nc;
             std::vector<int> rk(nc);
             hilbert_ranks(nx, ny, nz, rk.data());
             by_rank.resize(coff + nc);
@@ -1188,6 +1190,7 @@ class System : public SystemBase {
         d.cell_rep = crep;
         d.cell_by_rank = cbr;
         d.ncells = C;
+        d.rep_cells = (int)(nc2 / C);
         d.scan_part = part;
         const double rl = rc + sk;
         d.rlist2 = (T)(rl * rl);

@@ -1029,3 +1029,35 @@ def test_largest_handle_2_to_the_25_minus_1_particles():
     s.integrate(20, 0.002, 1.0, 1.0)
     assert s.error_word == 0 and s.step == 20
     s.close()
+
+
+@pytest.mark.parametrize("prec", [FP32, FP64])
+def test_batches_with_large_replicas_equal_standalone_runs(prec):
+    # replicas of more cells than a block scans for itself beside small ones, in
+    # every place of the batch: neighbours' cells are scanned together, whether or
+    # not both are being rebuilt; a handle of one replica bins in one launch
+    sizes = [(40, 50, 1), (400, 150, 2), (9, 37, 3), (400, 175, 4), (30, 60, 5)]
+    cases_ = [kg_case(nc, nb, seed=sd, jitter=0.05) for nc, nb, sd in sizes]
+
+    def batch(cs, seeds):
+        b = espp.System(precision=prec, replicas=[dict(box=c.cfg.box, n=c.cfg.n, types=c.cfg.types, bonds=c.cfg.bonds,
+                                                       seed=s) for c, s in zip(cs, seeds)])
+        b.set_wca()
+        b.set_fene()
+        b.set_resort_interval(25)
+        b.set_state(np.concatenate([c.cfg.x for c in cs]), np.concatenate([c.v for c in cs]),
+                    np.concatenate([c.cfg.img for c in cs]))
+        b.build_neighbors(WCA_RC, 0.4)
+        b.integrate(70, 0.005, 1.0, 1.0)
+        out = b.get_state()
+        assert b.error_word == 0 and b.n_rebuilds > 3
+        b.close()
+        return out
+
+    whole = batch(cases_, [90 + k for k in range(len(cases_))])
+    off = 0
+    for k, c in enumerate(cases_):
+        n = c.cfg.n
+        for a, q in zip(batch([c], [90 + k]), whole):
+            assert np.array_equal(a, q[off:off + n]), k
+        off += n
