@@ -451,7 +451,7 @@ __global__ void k_request_all(DevSys<T> s) {
 static inline int grid_for(int n, int block) { return (n + block - 1) / block; }
 
 // Blocks of the fused binning: four an SM are resident at once (its launch bounds).
-int binning_blocks() { return 4 * sm_count(); }
+int binning_blocks(int sms) { return 4 * sms; }
 
 // The fused binning has a block for every SCAN_THREADS particles, and for every
 // BIN_CELLS cells: in a dilute system the scan is most of its work.  us per step,
@@ -491,7 +491,7 @@ int Launch<T>::rebuild(const DevSys<T>& s, int cur, bool resort, bool permute_fo
     if (binning_fused(s)) {
         DevSys<T> a = s;
         void* args[] = {&a, &cur};
-        const int blocks = std::min(std::max(grid_for(s.N, SCAN_THREADS), grid_for(s.ncells, BIN_CELLS)), binning_blocks());
+        const int blocks = std::min(std::max(grid_for(s.N, SCAN_THREADS), grid_for(s.ncells, BIN_CELLS)), binning_blocks(s.sms));
         cudaLaunchCooperativeKernel((const void*)k_binning<T>, dim3(blocks), dim3(SCAN_THREADS), args, 0, st);
         launched = 1;
     } else {

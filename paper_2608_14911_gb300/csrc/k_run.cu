@@ -162,7 +162,7 @@ enum : int { RUN_NONE = 0, RUN_A, RUN_B };
 template <class T>
 static int run_form(const DevSys<T>& s) {
     if (!s.lj_fast || s.dpd || s.le_on || s.mlp_on || s.cells_mode) return RUN_NONE;
-    const int sms = sm_count();
+    const int sms = s.sms;
     if (sizeof(T) == 4) return s.ntiles <= 2 * sms ? RUN_A : s.ntiles <= 6 * sms ? RUN_B : RUN_NONE;
     if (4 * s.ntiles <= 3 * sms) return RUN_A;
     return s.ntiles <= 3 * sms && s.cap < 64 ? RUN_B : RUN_NONE;

@@ -103,6 +103,7 @@ template <class T> struct DevSys {
     int ntiles;
     const int* rep_tile_off;  // R + 1: first tile of each replica
     int* req;           // rebuild requested (per replica), set by the step kernel
+    int sms;            // SMs that the handle's kernels may count on (cooperative grids)
     // fault injection (tests): the barrier of k_binning, k_run whose wait runs out
     unsigned int bin_fault, run_fault;
     int* act;           // batches: the tiles of the replicas being rebuilt (ctrl->nact of them)
@@ -291,7 +292,7 @@ enum : int {
     MODE_FINAL = 3,   // F_s, v_s stored (end of an integrate call)
 };
 
-int binning_blocks();
+int binning_blocks(int sms);
 
 // ---- launchers (defined in the .cu files) ----------------------------------
 template <class T> struct Launch {

@@ -15,6 +15,7 @@
 #include <tuple>
 #include <vector>
 
+#include <cuda.h>
 #include <nvtx3/nvToolsExt.h>
 
 #include "h5md.h"
@@ -33,6 +34,42 @@ struct NvtxRange {
 
 void hilbert_ranks(int nx, int ny, int nz, int* rank);
 int scan_blocks_for(int ncells);
+
+// SMs that cooperative launches may count on: the device's, or fewer where the
+// stream, or the calling thread's context (whose graphs are captured), is a green
+// context with a part of them.
+static int usable_sms(cudaStream_t st) {
+    using GetCtx = CUresult(CUDAAPI*)(CUstream, CUcontext*, CUgreenCtx*);
+    using GetRes = CUresult(CUDAAPI*)(CUgreenCtx, CUdevResource*, CUdevResourceType);
+    struct Driver {
+        GetCtx get_ctx = nullptr;
+        GetRes get_res = nullptr;
+        Driver() {
+            void *a = nullptr, *b = nullptr;
+            const unsigned int v = 12050;  // the version that brought both
+            if (cudaGetDriverEntryPointByVersion("cuStreamGetCtx", &a, v, cudaEnableDefault) == cudaSuccess &&
+                cudaGetDriverEntryPointByVersion("cuGreenCtxGetDevResource", &b, v, cudaEnableDefault) == cudaSuccess &&
+                a && b) {
+                get_ctx = reinterpret_cast<GetCtx>(a);
+                get_res = reinterpret_cast<GetRes>(b);
+            }
+            (void)cudaGetLastError();
+        }
+    };
+    static const Driver drv;
+    int n = sm_count();
+    if (!drv.get_ctx) return n;
+    const CUstream streams[2] = {(CUstream)st, nullptr};
+    for (int k = 0; k < (st ? 2 : 1); ++k) {
+        CUcontext ctx = nullptr;
+        CUgreenCtx green = nullptr;
+        CUdevResource res;
+        if (drv.get_ctx(streams[k], &ctx, &green) == CUDA_SUCCESS && green &&
+            drv.get_res(green, &res, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS && res.sm.smCount > 0)
+            n = std::min(n, (int)res.sm.smCount);
+    }
+    return n;
+}
 
 #define CK(call)                                                                       \
     do {                                                                               \
@@ -61,6 +98,7 @@ struct SystemBase {
     virtual int mlp_train(const double* X, const double* Y, int nframes, int batch, int epochs, double lr,
                           uint64_t seed, double* loss_hist, float* grad_out) = 0;
     virtual int build_neighbors(double rc, double skin) = 0;
+    virtual void enter() = 0;
     virtual int get_neighbors(int64_t* row_ptr, int64_t* cols, int64_t cap) = 0;
     virtual int compute_forces(double* f, int where) = 0;
     virtual int integrate(int64_t nsteps, double dt, double gamma, double kT) = 0;
@@ -178,6 +216,14 @@ class System : public SystemBase {
         for (void* p : allocs) cudaFree(p);
         if (h_ctrl) cudaFreeHost(h_ctrl);
         if (h_back) cudaFreeHost(h_back);
+    }
+
+    // before every call: a handle used under another context captures its graphs anew
+    void enter() override {
+        const int n = usable_sms(st);
+        if (n == d.sms) return;
+        if (d.sms > 0) clear_graphs();
+        d.sms = n;
     }
 
     template <class P>
@@ -320,6 +366,7 @@ class System : public SystemBase {
             }
             rep_tile_off_h.push_back((int)tiles_h.size());
         }
+        enter();
         // pinned mirror and device buffers, after every check of the arguments
         CK(cudaMallocHost(&h_ctrl, sizeof(Ctrl)));
         int rc = ESPP_OK;
@@ -1175,7 +1222,7 @@ class System : public SystemBase {
         d.nscan_blocks = scan_blocks_for(C);
         if ((rc2 = alloc(&cnt, C, cell_allocs)) || (rc2 = alloc(&beg, C + 1, cell_allocs)) ||
             (rc2 = alloc(&rstart, C, cell_allocs)) || (rc2 = alloc(&crep, C, cell_allocs)) ||
-            (rc2 = alloc(&cbr, C, cell_allocs)) || (rc2 = alloc(&part, std::max(d.nscan_blocks, binning_blocks()), cell_allocs)))
+            (rc2 = alloc(&cbr, C, cell_allocs)) || (rc2 = alloc(&part, std::max(d.nscan_blocks, binning_blocks(sm_count())), cell_allocs)))
             return rc2;
         CK(cudaMemcpy(crep, rep_of.data(), C * sizeof(int), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(cbr, by_rank.data(), C * sizeof(int), cudaMemcpyHostToDevice));
@@ -2324,6 +2371,7 @@ static int guarded(espp_h h, F&& f) {
     // "last error" behind; drop it so launch checks see only our launches
     (void)cudaGetLastError();
     try {
+        h->impl->enter();
         return f(*h->impl);
     } catch (const std::exception& e) {
         h->impl->msg = e.what();

@@ -2,6 +2,8 @@
 same steps launched one kernel at a time: the same bits, at the sizes where
 its forms change and across list rebuilds, Hilbert resorts and calls of odd
 lengths; and a run it cannot finish reports what stopped it."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -200,3 +202,77 @@ def test_new_state_after_an_error_under_shear():
     (la, oa, fa), (lb, ob, fb) = out
     assert np.array_equal(la[0], lb[0]) and np.array_equal(la[1], lb[1])
     assert oa == ob and np.array_equal(fa, fb)
+
+
+class _Green:
+    """A green context of `sms` SMs (eight or the device's smallest part) with a
+    stream."""
+
+    class Res(ctypes.Structure):
+        _fields_ = [("type", ctypes.c_int), ("pad", ctypes.c_ubyte * 92), ("sm_count", ctypes.c_uint),
+                    ("rest", ctypes.c_ubyte * 44)]
+
+    def __init__(self):
+        import torch
+        torch.zeros(1, device="cuda")  # the device's primary context, current
+        self.cu = ctypes.CDLL("libcuda.so.1")
+        whole, part, rest = self.Res(), self.Res(), self.Res()
+        groups = ctypes.c_uint(1)
+        desc = ctypes.c_void_p()
+        self.green, self.ctx, self.stream = ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_void_p()
+        self.call("cuDeviceGetDevResource", 0, ctypes.byref(whole), 1)
+        self.call("cuDevSmResourceSplitByCount", ctypes.byref(part), ctypes.byref(groups), ctypes.byref(whole),
+                  ctypes.byref(rest), 0, 8)
+        self.call("cuDevResourceGenerateDesc", ctypes.byref(desc), ctypes.byref(part), 1)
+        self.call("cuGreenCtxCreate", ctypes.byref(self.green), desc, 0, 1)
+        self.call("cuCtxFromGreenCtx", ctypes.byref(self.ctx), self.green)
+        self.call("cuGreenCtxStreamCreate", ctypes.byref(self.stream), self.green, 1, 0)
+        self.sms = part.sm_count
+
+    def call(self, name, *args):
+        if not hasattr(self.cu, name):
+            pytest.skip("no green contexts: " + name)
+        rc = getattr(self.cu, name)(*args)
+        assert rc == 0, (name, rc)
+
+    def close(self):
+        self.call("cuStreamDestroy_v2", self.stream)
+        self.call("cuGreenCtxDestroy", self.green)
+
+
+@pytest.mark.parametrize("how", ["stream", "current"])
+@pytest.mark.parametrize("prec,chains,beads", [(FP32, 3, 43), (FP32, 40, 100), (FP32, 304, 128), (FP64, 3, 43),
+                                               (FP64, 40, 100), (FP64, 300, 200)])
+def test_a_part_of_the_sms(prec, chains, beads, how):
+    # the blocks of a cooperative launch fit at once on the SMs of its stream and of
+    # the context its graph was captured under, or the step graphs run
+    g = _Green()
+    assert g.sms < 64
+    c = I.kg_lattice(chains, beads, density=0.85, seed=4)
+
+    def go(stream):
+        s = espp.System(c.box, c.n, c.types, c.bonds, precision=prec, seed=4, stream=stream)
+        s.set_wca()
+        s.set_fene()
+        s.set_resort_interval(20)
+        s.set_state(c.x, I.maxwell_velocities(c.n, 1.0, seed=4), c.img)
+        s.build_neighbors(WCA_RC, 0.4)
+        for n in (33, 1, 20):
+            s.integrate(n, 0.005, 1.0, 1.0)
+        assert s.error_word == 0
+        out = s.get_state()
+        s.close()
+        return out
+
+    ref = go(0)
+    if how == "stream":
+        got = go(g.stream.value)
+    else:
+        g.call("cuCtxPushCurrent_v2", g.ctx)
+        try:
+            got = go(0)
+        finally:
+            g.call("cuCtxPopCurrent_v2", ctypes.byref(ctypes.c_void_p()))
+    g.close()
+    for p, q in zip(ref, got):
+        assert np.array_equal(p, q)
