@@ -1464,7 +1464,10 @@ class System : public SystemBase {
 
     // Small systems: one graph runs a whole segment of steps (k_run.cu): run,
     // then, while steps are left, rebuild and run again.
-    bool use_run() const { return chunk > 0 && !timing && Launch<T>::run_fits(d); }
+    // (a step shape that the caller or the tuner picked is the step kernel's)
+    bool use_run() const {
+        return chunk > 0 && !timing && (sizeof(T) == 8 || d.step_shape == 0) && Launch<T>::run_fits(d);
+    }
     int make_run(ChunkGraph** out) {
         auto key = std::make_tuple(0, 0, 0, 0);
         auto it = graphs.find(key);

@@ -9,7 +9,7 @@ import pytest
 
 from paper_2608_14911_gb300 import espp, inputs as I
 
-from _systems import WCA_RC
+from _systems import WCA_RC, kg_case
 
 pytestmark = pytest.mark.gpu
 FP32, FP64 = espp.ESPP_FP32, espp.ESPP_FP64
@@ -276,3 +276,47 @@ def test_a_part_of_the_sms(prec, chains, beads, how):
     g.close()
     for p, q in zip(ref, got):
         assert np.array_equal(p, q)
+
+
+def _integrate(case, prec, shape=0, chunk=64, timing=False, calls=(150,)):
+    """State after the calls, rebuilds, and kernel launches counted in them."""
+    s = case.system(prec, seed=8)
+    s.set_step_shape(shape)
+    s.set_graph_chunk(chunk)
+    s.set_kernel_timing(timing)
+    before = s.kernel_launches
+    for n in calls:
+        s.integrate(n, 0.005, 1.0, 1.0)
+    out = s.get_state(), s.n_rebuilds, s.kernel_launches - before
+    s.close()
+    return out
+
+
+@pytest.mark.parametrize("prec", [FP32, FP64])
+def test_step_graphs_equal_direct_launches(prec):
+    # graphs of the step kernel behind conditional rebuild nodes, of several step
+    # counts, on handles whose other runs stay in one kernel: a launch a step at least
+    case = kg_case()
+    ref, rebuilds, _ = _integrate(case, prec, chunk=0)
+    assert rebuilds > 4
+    forms = [dict(timing=True)] + [dict(shape=1)] * (prec == FP32)
+    for form in forms:
+        for chunk, calls in ((5, (150,)), (64, (1, 2, 20, 3, 124)), (7, (33, 117))):
+            got, rb, launches = _integrate(case, prec, chunk=chunk, calls=calls, **form)
+            assert launches >= 150 and rb == rebuilds, (form, chunk)
+            for a, b in zip(ref, got):
+                assert np.array_equal(a, b), (form, chunk)
+
+
+@pytest.mark.parametrize("shape", range(espp.STEP_SHAPES))
+def test_a_chosen_step_shape_is_the_step_kernels(shape):
+    # shape 0 leaves a small handle to the resident kernel, the others launch the
+    # step kernel in that shape: blocks of several tiles, the last one partial
+    case = kg_case(23, 56, seed=12, jitter=0.06)
+    ref, rebuilds, _ = _integrate(case, FP32, chunk=0)
+    got, rb, launches = _integrate(case, FP32, shape=shape)
+    assert rb == rebuilds and (launches >= 150) == (shape != 0)
+    for a, b in zip(ref, got):
+        assert np.array_equal(a, b)
+    # (FP64 handles have one shape)
+    assert _integrate(case, FP64, shape=shape)[2] < 150
