@@ -25,7 +25,7 @@ template <class T, int PPW, int GB, int MINB>
 __global__ void __launch_bounds__(TILE, MINB) k_run(DevSys<T> s, unsigned long long cond) {
     constexpr bool QUEUE = sizeof(T) == 8;
     constexpr int TPP = 32 / PPW;  // lanes per particle, blocks per tile
-    __shared__ __align__(16) unsigned char queue_mem[QUEUE ? sizeof(PairQueue<T, false, PPW>) * (TILE / 32) : 16];
+    extern __shared__ __align__(16) unsigned char queue_mem[];  // FP64: the warps' queues, up to 48 KB
     __shared__ long long stopped;
     Ctrl* c = s.ctrl;
     // what every block sees before any block can change it
@@ -183,13 +183,17 @@ cudaError_t Launch<T>::run(const DevSys<T>& s, unsigned long long cond, cudaStre
     const bool first = run_form(s) == RUN_A;
     const void* f;
     int blocks = s.ntiles;
+    size_t smem = 0;
     if constexpr (sizeof(T) == 4) {
         f = first ? (const void*)k_run<T, 32, 4, 2> : (const void*)k_run<T, 32, 2, 6>;
     } else {
         f = first ? (const void*)k_run<T, 8, 1, 3> : (const void*)k_run<T, 32, 1, 3>;
         if (first) blocks *= 4;
+        smem = (TILE / 32) * (first ? sizeof(PairQueue<T, false, 8>) : sizeof(PairQueue<T, false, 32>));
+        const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
     }
-    return cudaLaunchCooperativeKernel(f, dim3(blocks), dim3(TILE), args, 0, st);
+    return cudaLaunchCooperativeKernel(f, dim3(blocks), dim3(TILE), args, smem, st);
 }
 
 template bool Launch<float>::run_fits(const DevSys<float>&);

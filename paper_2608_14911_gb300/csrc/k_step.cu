@@ -119,9 +119,14 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
     const V4<T>* __restrict__ P = s.pos[cur];
     V4<T>* __restrict__ Pn = s.pos[cur ^ 1];
     const IntParams<T>* __restrict__ ip = s.ip;
-    __shared__ double red[ENERGY ? NPART : 1][ENERGY ? TILE + 4 : 1];
     static_assert(8 * NPART % 32 == 0 && 8 * NPART <= TILE, "whole warps reduce");
-    __shared__ __align__(16) unsigned char queue_mem[QUEUE ? sizeof(PairQueue<T, DPD, PPW>) * (TILE / 32) : 16];
+    // the warps' queues; after the forces the energy sums
+    constexpr size_t QUEUE_BYTES = QUEUE ? sizeof(PairQueue<T, DPD, PPW>) * (TILE / 32) : 16;
+    constexpr size_t RED_BYTES = ENERGY ? NPART * (TILE + 4) * sizeof(double) : 16;
+    constexpr size_t SMEM_BYTES = QUEUE_BYTES > RED_BYTES ? QUEUE_BYTES : RED_BYTES;
+    static_assert(SMEM_BYTES <= 48 * 1024, "static shared memory");
+    __shared__ __align__(16) unsigned char smem[SMEM_BYTES];
+    double (*red)[TILE + 4] = reinterpret_cast<double (*)[TILE + 4]>(smem);
 
     for (int t = t0; t < s.ntiles; t += TPP > 1 ? s.ntiles : gridDim.x * TPB) {
         const Tile tl = t == t0 ? tl0 : s.tiles[t];
@@ -167,7 +172,7 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
             if (!s.mlp_on && (FAST || !s.cells_mode)) {
                 const V4<T> xi = ld4<T>(P + i);
                 const int n = active ? s.nbr_cnt[i] : 0;
-                PairQueue<T, DPD, PPW>& q = reinterpret_cast<PairQueue<T, DPD, PPW>*>(queue_mem)[threadIdx.x >> 5];
+                PairQueue<T, DPD, PPW>& q = reinterpret_cast<PairQueue<T, DPD, PPW>*>(smem)[threadIdx.x >> 5];
                 const int ibase = tl.start + lt / PPW * PPW;
                 T rcmax2 = s.rc_max2;
                 if (DPD) rcmax2 = max(rcmax2, s.ip->dpd_rc2);
@@ -354,6 +359,7 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
             acc[P_BOND_LEN] = 0.5 * blen;
             acc[P_BOND_CNT] = 0.5 * bcnt;
             acc[P_VIR_XZ] = 0.5 * (double)vxz;
+            if (QUEUE) __syncthreads();  // every warp is done with its queue
             // eight threads per quantity add 16 particles each, then each other's
             // sums: a fifth of the FP64 additions of a tree over every warp
 #pragma unroll

@@ -49,7 +49,7 @@ __device__ __forceinline__ void queue_add(const Q& q, int k0, int k1, int sub, T
             fx = fma_rn(fr, dx, fx);
             fy = fma_rn(fr, dy, fy);
             fz = fma_rn(fr, dz, fz);
-            if (DPD) {
+            if constexpr (DPD) {
                 const T th = q.th[k];
                 fx = fma_rn(th, dx, fx);
                 fy = fma_rn(th, dy, fy);
@@ -61,7 +61,7 @@ __device__ __forceinline__ void queue_add(const Q& q, int k0, int k1, int sub, T
         for (int k = k0; k < k1; ++k) {
             const T dd = d[k];
             fx = fma_rn(q.fr[k], dd, fx);
-            if (DPD) fx = fma_rn(q.th[k], dd, fx);
+            if constexpr (DPD) fx = fma_rn(q.th[k], dd, fx);
         }
     }
 }

@@ -2,6 +2,8 @@
 // kernel: the Verlet list (thread per particle, or through the warp's pair
 // queue), the bonds and the Langevin thermostat.
 #pragma once
+#include <type_traits>
+
 #include "kernels.cuh"
 #include "packed.cuh"
 #include "pair_queue.cuh"
@@ -197,7 +199,7 @@ __device__ __forceinline__ void pair_loop(const DevSys<T>& s, const V4<T>* __res
 // fluid of 256,000 FP64 1241 / 822 us, DPD fluid of 786,432 FP32 446 / 323 us (215 M
 // warp instructions instead of 284 M, 26 of 32 lanes active instead of 11).
 template <class T, bool DPD, int PPW>
-struct PairQueue {
+struct PairQueueTerms {
     // list groups per block of the queue, terms held at a time.  FP32: small,
     // for the shared memory they take is L1 that the gathers lose (DPD fluid of
     // 786,432, step kernel: 4 / 128 320 us, 8 / 256 552 us, 4 / 64 329 us); FP64:
@@ -207,8 +209,14 @@ struct PairQueue {
     static constexpr int QR = sizeof(T) == 8 && !DPD ? 256 : 128;
     int col[QG * 4 * PPW];  // entries inside: row k of the particle's column
     T fr[QR], dx[QR], dy[QR], dz[QR];
-    T th[DPD ? QR : 1];     // the thermostat's term
 };
+// with the thermostat's term (FP64 without it: four warps' queues are 48 KB)
+template <class T, int PPW>
+struct PairQueueTh : PairQueueTerms<T, true, PPW> {
+    T th[PairQueueTerms<T, true, PPW>::QR];
+};
+template <class T, bool DPD, int PPW>
+using PairQueue = std::conditional_t<DPD, PairQueueTh<T, PPW>, PairQueueTerms<T, false, PPW>>;
 
 // PPW: particles per warp, 32 (one lane each) or 8 (four lanes share a
 // particle: lane t takes entry t of every group).  Returns the pair force on the
@@ -324,7 +332,7 @@ __device__ __forceinline__ void queue_loop(const DevSys<T>& s, const V4<T>* __re
                     Q.dx[b + lane] = dx;
                     Q.dy[b + lane] = dy;
                     Q.dz[b + lane] = dz;
-                    if (DPD) {
+                    if constexpr (DPD) {
                         T th = T(0);
                         if (less_nonneg(r2, s.ip->dpd_rc2)) {
                             DpdCtx<T> dc;
