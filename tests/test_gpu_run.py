@@ -320,3 +320,30 @@ def test_a_chosen_step_shape_is_the_step_kernels(shape):
         assert np.array_equal(a, b)
     # (FP64 handles have one shape)
     assert _integrate(case, FP64, shape=shape)[2] < 150
+
+
+@pytest.mark.parametrize("prec,tol", [(FP32, 2e-4), (FP64, 1e-11)])
+def test_list_overflow_inside_a_resident_run(prec, tol, monkeypatch):
+    # a dilute gas drawn together: its lists outgrow their capacity some rebuilds
+    # into one call, which grows them and goes on from the step it had reached.
+    # (The order of storage and of the sums is another afterwards: rounding only,
+    # over 100 steps without many collisions; coordinates of 40 sigma)
+    g = np.random.default_rng(3)
+    k = np.arange(512)
+    x = I.f32(20.0 + 2.2 * (np.stack([k % 8, k // 8 % 8, k // 64], 1) - 3.5) + g.uniform(-0.2, 0.2, (512, 3)))
+    v = -0.9 * (x - 20.0)
+    out = []
+    for cap in (256, 8):
+        monkeypatch.setenv("ESPP_FAULT_LIST_CAP", str(cap))
+        s = espp.System((40.0, 40.0, 40.0), 512, None, None, precision=prec, seed=4)
+        s.set_lj(1.0, 1.0, 1.5)
+        s.set_state(x, v, None)
+        s.build_neighbors(1.5, 0.4)
+        assert s.list_capacity == cap  # (the first lists fit)
+        s.integrate(100, 0.005, 0.0, 0.0)
+        assert s.error_word == 0 and s.step == 100 and s.n_rebuilds > 5
+        assert (s.list_capacity > cap) == (cap == 8)
+        out.append(s.get_state())
+        s.close()
+    for a, b in zip(*out):
+        assert np.abs(a - b).max() <= tol

@@ -121,3 +121,47 @@ def test_dilute_boxes(prec, tol, band, n, box):
     m = O.Model(1, {(0, 0): ("lj_capped", 1.0, 1.0, 1.1, True, 0.8)}, None)
     fo, _ = O.forces(m, c.box, c.x, c.types, c.bonds)
     assert rel_rms(f, fo) <= tol
+
+
+@pytest.mark.parametrize("prec,n_chains", [(FP32, 40), (FP32, 90), (FP64, 40), (FP64, 330)])
+@pytest.mark.parametrize("w", [1, 2, 3])
+@pytest.mark.parametrize("variant", ["lees_edwards", "exclusions"])
+def test_sheared_and_excluded_lists(prec, n_chains, w, variant):
+    # the search's other instances, a team of lanes and one thread per particle,
+    # against the oracle.  FP32 under shear: the offset and each of the three
+    # differences it enters are rounded at up to 32 sigma, 1e-6 each
+    c = I.kg_lattice(n_chains, 100, density=0.85, seed=5, jitter=0.1)
+    le = variant == "lees_edwards"
+    shear, t = 0.4, 3.3
+    s = espp.System(c.box, c.n, c.types, c.bonds, precision=prec, seed=3)
+    s.set_wca()
+    s.set_fene()
+    s.set_cell_subdivision(w)
+    if le:
+        s.set_lees_edwards(True, shear, t)
+    else:
+        s.set_exclude_bonded(True)
+    s.set_state(c.x, None, c.img)
+    s.build_neighbors(1.1225, RL - 1.1225)
+    row, cols = s.get_neighbors()
+    s.close()
+    O.set_lees_edwards(le, shear)
+    try:
+        orow, ocols = O.neighbors(c.box, c.x, RL, time=t if le else 0.0)
+    finally:
+        O.set_lees_edwards(False)
+    i = np.repeat(np.arange(c.n), np.diff(orow))
+    want = i * c.n + ocols
+    if not le:
+        b = np.asarray(c.bonds)
+        want = np.setdiff1d(want, np.concatenate([b[:, 0] * c.n + b[:, 1], b[:, 1] * c.n + b[:, 0]]))
+    got = np.repeat(np.arange(c.n), np.diff(row)) * c.n + cols
+    assert len(np.unique(got)) == len(got)
+    delta = shear * c.box[2] * t if le else 0.0
+    for q in np.setxor1d(got, want):
+        d = c.x[q // c.n] - c.x[q % c.n]
+        k = np.rint(d[2] / c.box[2])
+        d[2] -= k * c.box[2]
+        d[0] -= k * delta
+        d -= c.box * np.rint(d / c.box)
+        assert abs(np.linalg.norm(d) - RL) <= (0.0 if prec == FP64 else 1e-5 if le else 1e-6), (q // c.n, q % c.n)
