@@ -98,7 +98,6 @@ struct SystemBase {
     virtual int mlp_train(const double* X, const double* Y, int nframes, int batch, int epochs, double lr,
                           uint64_t seed, double* loss_hist, float* grad_out) = 0;
     virtual int build_neighbors(double rc, double skin) = 0;
-    virtual void enter() = 0;
     virtual int get_neighbors(int64_t* row_ptr, int64_t* cols, int64_t cap) = 0;
     virtual int compute_forces(double* f, int where) = 0;
     virtual int integrate(int64_t nsteps, double dt, double gamma, double kT) = 0;
@@ -218,8 +217,10 @@ class System : public SystemBase {
         if (h_back) cudaFreeHost(h_back);
     }
 
-    // before every call: a handle used under another context captures its graphs anew
-    void enter() override {
+    // Before cooperative launches and their capture: a handle used under another
+    // context captures its graphs anew.  (Two driver queries: once a host call
+    // that launches such kernels, not in every call.)
+    void count_sms() {
         const int n = usable_sms(st);
         if (n == d.sms) return;
         if (d.sms > 0) clear_graphs();
@@ -366,7 +367,6 @@ class System : public SystemBase {
             }
             rep_tile_off_h.push_back((int)tiles_h.size());
         }
-        enter();
         // pinned mirror and device buffers, after every check of the arguments
         CK(cudaMallocHost(&h_ctrl, sizeof(Ctrl)));
         int rc = ESPP_OK;
@@ -1261,6 +1261,7 @@ class System : public SystemBase {
     int rebuild_now(bool permute_force, bool resort = true) {
         NvtxRange nvtx_range("espp_rebuild");
         if (!cells_ready) return fail(ESPP_ERR_STATE, "call espp_build_neighbors first");
+        count_sms();
         for (int attempt = 0; attempt < 6; ++attempt) {
             touch();
             launches += Launch<T>::rebuild(d, cur, resort, permute_force, st);
@@ -1601,6 +1602,7 @@ class System : public SystemBase {
             return fail(ESPP_ERR_ARG, "the DPD cutoff exceeds the list cutoff");
         rcode = upload_int_params(dt, gamma, kT);
         if (rcode) return rcode;
+        count_sms();
         rcode = prepare_graphs();
         if (rcode) return rcode;
         const int64_t step0 = c0.step;
@@ -1968,6 +1970,7 @@ class System : public SystemBase {
         // it from them (buffer 1 holds a copy), without a resort
         // (list-free mode: bin the saved positions, which the last step binned)
         touch();
+        count_sms();
         Launch<T>::request_all(d, st);
         launches += 1 + Launch<T>::rebuild(d, d.cells_mode ? 0 : 1, false, false, st);
         CK(cudaGetLastError());
@@ -2374,7 +2377,6 @@ static int guarded(espp_h h, F&& f) {
     // "last error" behind; drop it so launch checks see only our launches
     (void)cudaGetLastError();
     try {
-        h->impl->enter();
         return f(*h->impl);
     } catch (const std::exception& e) {
         h->impl->msg = e.what();
