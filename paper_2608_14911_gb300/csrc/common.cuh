@@ -83,13 +83,16 @@ __device__ __forceinline__ T drift(T x, T v, T dt) {
 // ---------------------------------------------------------------------------
 // Comparisons that keep FP64 off its unit (a double compare occupies it like an
 // addition; GB300 has two FP64 lanes per SM): non-negative doubles order as
-// their bit patterns, a NaN compares false as it does in floating point.
+// their bit patterns, in which a NaN lies above every number.
 // ---------------------------------------------------------------------------
+// a < b.  A NaN as a compares false; as b it compares true for doubles and false for
+// floats (a displacement's square, the one computed b, is of finite coordinates).
 __device__ __forceinline__ bool less_nonneg(float a, float b) { return a < b; }
 __device__ __forceinline__ bool less_nonneg(double a, double b) {
     return (unsigned long long)__double_as_longlong(a) < (unsigned long long)__double_as_longlong(b);
 }
-// |a| > b for b >= 0 (a NaN counts as larger)
+// |a| > b for b >= 0 (a NaN compares true for doubles, false for floats: both ways
+// min_image returns it)
 __device__ __forceinline__ bool abs_greater(float a, float b) { return fabsf(a) > b; }
 __device__ __forceinline__ bool abs_greater(double a, double b) {
     return (unsigned long long)(__double_as_longlong(a) & 0x7fffffffffffffffll) >

@@ -157,7 +157,10 @@ __global__ void k_run_begin(DevSys<T> s, long long target, int final_step, int b
 // graphs / resident, rebuilds included: KG melt FP32 1,000 17.2 / 8.4, 5,000 17.9 /
 // 9.7, 40,000 18.7 / 11.5, 110,000 23 / 16.6; LJ fluid FP32 4,000 26.9 / 17.1, 27,436
 // 34.3 / 25.0, 108,000 44.6 / 39.7; KG melt FP64 1,000 24.0 / 15.8, 10,000 33.9 / 25.5,
-// 40,000 47.6 / 39.6.
+// 40,000 47.6 / 39.6.  Batches take them by the same rule, though some replica of a
+// large one ends the kernel at nearly every step: FP32 2 x 1,000 beads 18.5 / 9.9, 64 x
+// 1,000 50.9 / 49.1, 16 x 5,000 45.6 / 44.5; FP64 2 x 1,000 26.1 / 17.8, 64 x 1,000 94.2 /
+// 93.4, 16 x 5,000 99.0 / 99.0.
 enum : int { RUN_NONE = 0, RUN_A, RUN_B };
 template <class T>
 static int run_form(const DevSys<T>& s) {

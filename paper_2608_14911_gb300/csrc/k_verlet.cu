@@ -12,10 +12,10 @@
 // has no hit branch: a hit is one predicated store of the entry into the lane's
 // column of shared memory (conflict-free: the column is the bank), and the
 // columns are written out as whole int4 groups, all lanes together, when they
-// fill and at the end.  KG melt, 1M beads, FP32, whole cells: 131 us a build,
-// 90.8 M warp instructions, 21 of 32 lanes active (with the hit branch 220 us,
-// 172.6 M, 14); LJ fluid, 4.2M, half cells: 1.9 ms (3.1 ms).  What is left is
-// half issue (55%) and half the L1 data pipe (68%: each candidate is a 16-byte
+// fill and at the end.  KG melt, 1M beads, FP32, whole cells: 138 us a build under
+// ncu, 95.0 M warp instructions, 23 of 32 lanes active (with the hit branch 226 us,
+// 172.6 M, 14); LJ fluid, 4.2M, half cells: 1.8 ms (3.1 ms).  What is left is
+// half issue (54%) and half the L1 data pipe (64%: each candidate is a 16-byte
 // gather of its own).
 //
 // FP64 handles test the candidates in FP32, on float copies of the entries; a

@@ -61,7 +61,7 @@ __device__ __forceinline__ void pair_loop(const DevSys<T>& s, const V4<T>* __res
     // the groups of the next batch are requested before the positions of the
     // current one, so their latency overlaps the current batch; the first
     // batch is read without waiting for the count (groups past the count are
-    // allocated, and dropped whole; the last group is padded with -1)
+    // allocated, and dropped whole)
     // padding entries (the rest of the last group, and whole groups past the
     // count) name the padding slot, whose position is far outside the box:
     // every entry is loaded and evaluated without a test of its own
@@ -195,16 +195,16 @@ __device__ __forceinline__ void pair_loop(const DevSys<T>& s, const V4<T>* __res
 // keeps the entries inside, then evaluates the warp's entries 32 at a time, one
 // per lane whoever owns them, the exact test included, into shared memory; every
 // particle then adds its own terms in list order, as a walk of the list would.
-// Step kernel, walking its own list / queue: KG melt of 1M FP64 876 / 464 us, LJ
-// fluid of 256,000 FP64 1241 / 822 us, DPD fluid of 786,432 FP32 446 / 323 us (215 M
+// Step kernel, walking its own list / queue: KG melt of 1M FP64 876 / 458 us, LJ
+// fluid of 256,000 FP64 1241 / 822 us, DPD fluid of 786,432 FP32 446 / 301 us (215 M
 // warp instructions instead of 284 M, 26 of 32 lanes active instead of 11).
 template <class T, bool DPD, int PPW>
 struct PairQueueTerms {
     // list groups per block of the queue, terms held at a time.  FP32: small,
     // for the shared memory they take is L1 that the gathers lose (DPD fluid of
-    // 786,432, step kernel: 4 / 128 320 us, 8 / 256 552 us, 4 / 64 329 us); FP64:
+    // 786,432, step kernel: 4 / 128 301 us, 8 / 256 377 us, 4 / 64 303 us); FP64:
     // large, for every stretch of terms costs its particles' additions once
-    // more (KG melt of 1M: 8 / 256 530 us, 4 / 128 570 us, 4 / 64 609 us)
+    // more (KG melt of 1M: 8 / 256 458 us, 4 / 128 493 us, 4 / 64 527 us)
     static constexpr int QG = sizeof(T) == 8 ? 8 : 4;
     static constexpr int QR = sizeof(T) == 8 && !DPD ? 256 : 128;
     int col[QG * 4 * PPW];  // entries inside: row k of the particle's column
