@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? ESPP_CF_MINB32 : 4) k_c
                             dc.seed = g.seed;
                             dc.step = step;
                             dc.le_vs = LE ? (T)(s.le_shear * (double)g.L[2]) : T(0);
-                            th = dpd_value<T>(s.ip, dc, dx, dy, dz, r2, ld4<T>(VE + ej), nz);
+                            th = dpd_value<T, LE>(s.ip, dc, dx, dy, dz, r2, ld4<T>(VE + ej), nz);
                         }
                         Q.th[b + lane] = th;
                     }

@@ -76,7 +76,7 @@ __device__ __forceinline__ void dpd_loop(const DevSys<T>& s, const V4<T>* __rest
             const T dz = shifted_diff(xi.z, zim, xj.z, L2, code >> 4);
             const T r2 = dx * dx + dy * dy + dz * dz;
             if (!(r2 < rc2)) continue;
-            dpd_term<T>(ip, c, dx, dy, dz, r2, ld4<T>(VS + j), fx, fy, fz, nz);
+            dpd_term<T, LE>(ip, c, dx, dy, dz, r2, ld4<T>(VS + j), fx, fy, fz, nz);
         }
     }
 }
@@ -92,8 +92,9 @@ __global__ void __launch_bounds__(TILE) k_vsnap(DevSys<T> s) {
 }
 
 // SH: launch shape (STEP_SHAPES) of the plain FP32 list path.  PPW: particles
-// per warp of the queue path (32, or 8 with four lanes per particle).
-template <class T, int MODE, bool ENERGY, bool FAST, bool DPD, bool LE, int SH = 0, int PPW = 32>
+// per warp of the queue path (32, or 8 with four lanes per particle).  WALK: FP32
+// DPD walks the lists instead (see step_walks).
+template <class T, int MODE, bool ENERGY, bool FAST, bool DPD, bool LE, int SH = 0, int PPW = 32, bool WALK = false>
 __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
                                   sizeof(T) == 4 ? (DPD ? ESPP_STEP_MINB32_DPD
                                                         : (SH == 0 ? ESPP_STEP_MINB32 : STEP_SHAPES[SH].minb))
@@ -104,7 +105,7 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
     constexpr int TPB = STEP_SHAPES[SH].tpb;
     static_assert(TPB == 1 || !ENERGY, "energy reductions take one tile per block");
     static_assert(PPW == 32 || (TPB == 1 && !ENERGY), "four lanes per particle: single tiles, no reductions");
-    constexpr bool QUEUE = sizeof(T) == 8 || DPD;
+    constexpr bool QUEUE = (sizeof(T) == 8 || DPD) && !WALK;
     constexpr int TPP = 32 / PPW;  // lanes per particle, blocks per tile
     // index inside the tile
     const int lt = TPP > 1 ? (int)(blockIdx.x % TPP) * (TILE / TPP) + (int)threadIdx.x / TPP
@@ -252,6 +253,13 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
                     vxz = w.y;
                 }
             } else if constexpr (!QUEUE) {
+                DpdCtx<T> dc;
+                if constexpr (DPD) {
+                    dc.vi = s.vel[i];
+                    dc.seed = g.seed;
+                    dc.step = step;
+                    dc.le_vs = le.vs;
+                }
                 if (FAST) {
                     PairRec<T> pr;
                     pr.rc2 = s.pair[0].rc2;
@@ -261,16 +269,16 @@ __global__ void __launch_bounds__(TILE * STEP_SHAPES[SH].tpb,
                         pr.eps4 = s.pair[0].eps4;
                         pr.shift = s.pair[0].shift;
                     }
-                    pair_loop<T, ENERGY, false, true, LE, STEP_SHAPES[SH].groups>(s, P, i, n, xi, ti, &pr, L0, L1, L2, fx,
-                                                                                  fy, fz, pe, vir, vxz, &le);
+                    pair_loop<T, ENERGY, false, true, LE, STEP_SHAPES[SH].groups, false, DPD>(
+                        s, P, i, n, xi, ti, &pr, L0, L1, L2, fx, fy, fz, pe, vir, vxz, &le, &dc);
                 } else if (s.ntypes == 1) {
                     const PairRec<T> pr = s.pair[0];
-                    if (pr.kind != 0)
-                        pair_loop<T, ENERGY, false, false, LE>(s, P, i, n, xi, ti, &pr, L0, L1, L2, fx, fy, fz, pe, vir,
-                                                               vxz, &le);
+                    if (DPD || pr.kind != 0)
+                        pair_loop<T, ENERGY, false, false, LE, 1, false, DPD>(s, P, i, n, xi, ti, &pr, L0, L1, L2, fx, fy,
+                                                                              fz, pe, vir, vxz, &le, &dc);
                 } else {
-                    pair_loop<T, ENERGY, true, false, LE>(s, P, i, n, xi, ti, nullptr, L0, L1, L2, fx, fy, fz, pe, vir,
-                                                          vxz, &le);
+                    pair_loop<T, ENERGY, true, false, LE, 1, false, DPD>(s, P, i, n, xi, ti, nullptr, L0, L1, L2, fx, fy,
+                                                                         fz, pe, vir, vxz, &le, &dc);
                 }
             }
             if (LATE_VEL) {
@@ -471,6 +479,32 @@ static bool queue_spread(const DevSys<T>& s) {
     return s.N < 49152;
 }
 
+// FP32 handles with the DPD thermostat and one lane per particle walk their lists
+// (pair_loop, the thermostat's term where it is met) instead of taking the queue
+// where the queue has little to save: few entries inside the thermostat's cutoff
+// (its term then runs rarely, and every other entry would pass through shared memory
+// for a Lennard-Jones term), or most entries inside some cutoff.  The fractions are
+// those of a uniform density outside the potentials' cores (0.9 sigma).  Step kernel
+// (event-timed), queue / walk, thermostat inside x, any cutoff inside y of the list:
+//   LJ 2.5, skin 0.3, DPD 1.0 (0.01, 0.70): 55,000 54.5 / 33.5 us, 256,000 172 / 74, 780,000
+//     469 / 180; two types 256,000 184 / 115; under shear 187 / 93
+//   LJ 2.5, skin 1.0, DPD 1.0 (0.01, 0.35): 256,000 214 / 126
+//   LJ 2.5, skin 0.3, DPD 1.5 (0.12, 0.70): 55,000 72.7 / 67.9, 256,000 218 / 167
+//   the same, DPD 2.5 (0.70, 0.70): 55,000 75.7 / 81.6, 256,000 226 / 206
+//   table 1.5, skin 0.05, DPD 1.5 (0.90, 0.90): 256,000 69 / 64
+//   table 1.5, skin 0.4, DPD 1.0 (0.15, 0.49): 256,000 73 / 75
+//   LJ 2.5, skin 1.0, DPD 2.0 (0.17, 0.35): 256,000 267 / 313
+//   WCA, skin 0.4, DPD 1.1 (0.21, 0.25): 256,000 35.5 / 46.9
+//   table 1.0, skin 0.6, DPD 1.0 (0.24, 0.24): 256,000 95 / 163
+template <class T>
+static bool step_walks(const DevSys<T>& s) {
+    if (sizeof(T) == 8) return false;
+    const double core = s.pair_core3, list = pow((double)s.rlist2, 1.5) - core;
+    const double dpd = pow((double)s.dpd_rc2, 1.5) - core;
+    const double any = pow((double)(s.dpd_rc2 > s.rc_max2 ? s.dpd_rc2 : s.rc_max2), 1.5) - core;
+    return dpd < 0.1 * list || (any > 0.65 * list && s.N >= 131072);
+}
+
 template <class T>
 int Launch<T>::step(const DevSys<T>& s, int mode, bool energy, int cur, double* f_out,
                     unsigned long long next_cond, int grid, cudaStream_t st) {
@@ -489,11 +523,18 @@ int Launch<T>::step(const DevSys<T>& s, int mode, bool energy, int cur, double* 
                     (mode == MODE_STEP || mode == MODE_FINAL) && !dpd) ? s.step_shape : 0;
     // queue path of a small handle: four lanes per particle (see the rule above)
     const bool spread = (sizeof(T) == 8 || dpd) && !s.mlp_on && !s.cells_mode && queue_spread(s);
+    const bool walk = dpd && !spread && !s.mlp_on && !s.cells_mode && step_walks(s);
 #define ESPP_STEP_Q(M, E, F, D, LE)                                                                        \
     do {                                                                                                   \
         if constexpr ((sizeof(T) == 8 || (D)) && !(E)) {                                                   \
             if (spread) {                                                                                  \
                 k_step<T, M, E, F, D, LE, 0, 8><<<4 * s.ntiles, TILE, 0, st>>>(s, cur, f_out, next_cond);  \
+                break;                                                                                     \
+            }                                                                                              \
+        }                                                                                                  \
+        if constexpr (sizeof(T) == 4 && (D)) {                                                             \
+            if (walk) {                                                                                    \
+                k_step<T, M, E, F, D, LE, 0, 32, true><<<gr, TILE, 0, st>>>(s, cur, f_out, next_cond);     \
                 break;                                                                                     \
             }                                                                                              \
         }                                                                                                  \

@@ -158,6 +158,8 @@ template <class T> struct DevSys {
     int N;
     BondRec<T> bond;
     T rc_max2;          // largest pair cutoff^2
+    T dpd_rc2;          // DPD cutoff^2 (host rules)
+    double pair_core3;  // (0.9 sigma)^3 of the smallest Lennard-Jones core, 0 where a pair has none (host rules)
     T rlist2;           // (rc + skin)^2
     T half_skin2;       // (skin / 2)^2
     T skin;

@@ -105,22 +105,26 @@ struct DpdCtx {
 // in the pair, so both sides add exactly opposite forces.  nz: the partner is
 // the image above (+1) or below (-1) a sheared face (Lees-Edwards), whose
 // velocity is vj + nz le_shear Lz along x.  dpd_value is the magnitude
-// divided by r (the force on i is dpd_value * d).
-template <class T>
+// divided by r (the force on i is dpd_value * d).  Its sums are written as the fused
+// operations they round as: every kernel that evaluates a pair, whatever the
+// compiler would contract in it, gets the same bits.
+template <class T, bool LE>
 __device__ __forceinline__ T dpd_value(const IntParams<T>* __restrict__ ip, const DpdCtx<T>& c, T dx, T dy, T dz,
                                        T r2, const V4<T>& vj, int nz = 0) {
     const T r = sqrt(r2), inv_r = T(1) / r;
     const T w = T(1) - r * ip->dpd_inv_rc;
     const T vjx = nz == 0 ? vj.x : vj.x + (T)nz * c.le_vs;
-    const T ev = (dx * (c.vi.x - vjx) + dy * (c.vi.y - vj.y) + dz * (c.vi.z - vj.z)) * inv_r;
+    const T ex = c.vi.x - vjx, ey = c.vi.y - vj.y, ez = c.vi.z - vj.z;
+    const T exy = LE ? fma_rn(dy, ey, mul_rn(dx, ex)) : fma_rn(dx, ex, mul_rn(dy, ey));
+    const T ev = fma_rn(dz, ez, exy) * inv_r;
     const T th = dpd_theta<T>(c.seed, bits_as_int(c.vi.w), bits_as_int(vj.w), c.step);
-    return (-ip->gamma * w * w * ev + ip->dpd_amp * w * th) * inv_r;
+    return fma_rn(ip->dpd_amp * w, th, mul_rn(-ip->gamma * w * w, ev)) * inv_r;
 }
 
-template <class T>
+template <class T, bool LE>
 __device__ __forceinline__ void dpd_term(const IntParams<T>* __restrict__ ip, const DpdCtx<T>& c, T dx, T dy,
                                          T dz, T r2, const V4<T>& vj, T& fx, T& fy, T& fz, int nz = 0) {
-    const T val = dpd_value<T>(ip, c, dx, dy, dz, r2, vj, nz);
+    const T val = dpd_value<T, LE>(ip, c, dx, dy, dz, r2, vj, nz);
     fx += val * dx;
     fy += val * dy;
     fz += val * dz;

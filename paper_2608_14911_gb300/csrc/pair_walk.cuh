@@ -44,14 +44,15 @@ __device__ __forceinline__ V4<T> ldp(const V4<T>* p) {
 // read in batches of int4 groups: all indices of a batch first, then all
 // neighbour positions, then the arithmetic, so that each thread keeps several
 // independent loads in flight; the next batch's indices are prefetched.
-// (FP32 without DPD; FP64 handles and the DPD thermostat take queue_loop.)
+// (FP64 handles, and the DPD thermostat but where step_walks says so, take
+// queue_loop; the thermostat's terms follow each pair's force here as there.)
 // Entries with x code 3 cross a sheared face (Lees-Edwards): their x
 // difference is taken from the current offset in *le.
-template <class T, bool ENERGY, bool MULTI, bool FAST, bool LE, int GB32 = 1, bool COH = false>
+template <class T, bool ENERGY, bool MULTI, bool FAST, bool LE, int GB32 = 1, bool COH = false, bool DPD = false>
 __device__ __forceinline__ void pair_loop(const DevSys<T>& s, const V4<T>* __restrict__ P, int i, int n,
                                           const V4<T>& xi, int ti, const PairRec<T>* pr1,
                                           T L0, T L1, T L2, T& fx, T& fy, T& fz, T& pe, T& vir, T& vxz,
-                                          const LeCtx<T>* le) {
+                                          const LeCtx<T>* le, const DpdCtx<T>* dc = nullptr) {
     const T xim = xi.x - L0, yim = xi.y - L1, zim = xi.z - L2;
     constexpr int GB = GB32;  // int4 groups per batch
     const int ng = (n + 3) >> 2;
@@ -69,7 +70,7 @@ __device__ __forceinline__ void pair_loop(const DevSys<T>& s, const V4<T>* __res
     const int4 pad4 = make_int4(pad, pad, pad, pad);
     // FP32 single-type Lennard-Jones without energies (the step's hot path):
     // two entries per packed FP32x2 instruction, forces summed in two lanes
-    constexpr bool PACK = FAST && !ENERGY;
+    constexpr bool PACK = FAST && !ENERGY && !DPD;
     f32x2 px = 0ull, py = 0ull, pz = 0ull;
     f32x2 xi2 = 0ull, yi2 = 0ull, zi2 = 0ull, sg2 = 0ull, e24 = 0ull;
     if constexpr (PACK) {
@@ -157,20 +158,33 @@ __device__ __forceinline__ void pair_loop(const DevSys<T>& s, const V4<T>* __res
                 const T dx = xi.x - xj[q].x, dy = xi.y - xj[q].y, dz = xi.z - xj[q].z;
                 pair_term<T, ENERGY, MULTI, FAST>(s, ti, pr1, dx, dy, dz, bits_as_int(xj[q].w), fx, fy, fz, pe,
                                                   vir, vxz);
+                if constexpr (DPD) {
+                    const T r2 = dx * dx + dy * dy + dz * dz;
+                    if (r2 < s.ip->dpd_rc2)
+                        dpd_term<T, LE>(s.ip, *dc, dx, dy, dz, r2, ld4<T>(s.vsnap + nbr_slot(jj[q])), fx, fy, fz);
+                }
             }
         } else {
 #pragma unroll
             for (int q = 0; q < 4 * GB; ++q) {
                 const int code = nbr_code(jj[q]);
+                int nz = 0;
                 T dx;
-                if (LE && (code & 3) == 3)
-                    dx = le_dx(xi.x, xj[q].x, (code >> 4) == 1 ? 1 : -1, le->d, L0, le->inv_Lx);
-                else
+                if (LE && (code & 3) == 3) {
+                    nz = (code >> 4) == 1 ? 1 : -1;
+                    dx = le_dx(xi.x, xj[q].x, nz, le->d, L0, le->inv_Lx);
+                } else {
                     dx = shifted_diff(xi.x, xim, xj[q].x, L0, code & 3);
+                }
                 const T dy = shifted_diff(xi.y, yim, xj[q].y, L1, (code >> 2) & 3);
                 const T dz = shifted_diff(xi.z, zim, xj[q].z, L2, code >> 4);
                 pair_term<T, ENERGY, MULTI, FAST>(s, ti, pr1, dx, dy, dz, bits_as_int(xj[q].w), fx, fy, fz,
                                                   pe, vir, vxz);
+                if constexpr (DPD) {
+                    const T r2 = dx * dx + dy * dy + dz * dz;
+                    if (r2 < s.ip->dpd_rc2)
+                        dpd_term<T, LE>(s.ip, *dc, dx, dy, dz, r2, ld4<T>(s.vsnap + nbr_slot(jj[q])), fx, fy, fz, nz);
+                }
             }
         }
     }
@@ -340,7 +354,7 @@ __device__ __forceinline__ void queue_loop(const DevSys<T>& s, const V4<T>* __re
                             dc.seed = g.seed;
                             dc.step = step;
                             dc.le_vs = le.vs;
-                            th = dpd_value<T>(s.ip, dc, dx, dy, dz, r2, ld4<T>(s.vsnap + j), nz);
+                            th = dpd_value<T, LE>(s.ip, dc, dx, dy, dz, r2, ld4<T>(s.vsnap + j), nz);
                         }
                         Q.th[b + lane] = th;
                     }

@@ -570,7 +570,12 @@ class System : public SystemBase {
         d.lj_fast = (!d.cells_mode && ntypes == 1 && pair_h[0][0].kind == ESPP_LJ) ? 1 : 0;
         d.mlp_on = (pair_h[0][0].kind == ESPP_MLP) ? 1 : 0;
         d.rc_max2 = T(0);
-        for (int k = 0; k < ntypes * ntypes; ++k) d.rc_max2 = std::max(d.rc_max2, pr[k].rc2);
+        double sig2 = INFINITY;
+        for (int k = 0; k < ntypes * ntypes; ++k) {
+            d.rc_max2 = std::max(d.rc_max2, pr[k].rc2);
+            sig2 = std::min(sig2, pr[k].kind == ESPP_LJ ? (double)pr[k].sig2 : 0.0);
+        }
+        d.pair_core3 = std::pow(0.81 * sig2, 1.5);
         if (d.mlp_on && !mlp_bits.empty()) {
             MlpWeights w;
             memset(&w, 0, sizeof(w));
@@ -2039,6 +2044,7 @@ class System : public SystemBase {
             }
             d.dpd = 1;
             dpd_rc = rc;
+            d.dpd_rc2 = (T)(rc * rc);
         } else {
             return fail(ESPP_ERR_ARG, "unknown thermostat kind");
         }

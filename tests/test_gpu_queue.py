@@ -119,3 +119,38 @@ def test_cell_forces_spread_does_not_change_the_bits(prec):
         s.close()
     for a, b, both in zip(*out):
         assert np.array_equal(np.concatenate([a, b]), both)
+
+
+@pytest.mark.parametrize("le", [False, True])
+@pytest.mark.parametrize("types,pair", [(1, "lj"), (1, "capped"), (2, "lj")])
+def test_dpd_walk_does_not_change_the_bits(types, pair, le):
+    # long lists with few entries inside the thermostat's cutoff: each replica alone
+    # takes the queue (four lanes per particle), both together walk their lists
+    m = 19
+    c0 = I.lj_fcc(m, m, m, density=0.8442)
+    cs = []
+    for seed in (3, 4):
+        g = np.random.default_rng(seed)
+        x = I.f32(np.mod(c0.x + g.uniform(-0.06, 0.06, c0.x.shape), c0.box))
+        x[x >= c0.box] = 0.0
+        cs.append((x, I.maxwell_velocities(c0.n, 0.72, seed=seed)))
+    t = (np.arange(c0.n) % types).astype(np.int32)
+    out = []
+    for group in ([cs[0]], [cs[1]], cs):
+        s = espp.System(precision=FP32, replicas=[dict(box=c0.box, n=c0.n, types=t, bonds=None, seed=9) for _ in group])
+        for a in range(types):
+            for b in range(a, types):
+                if pair == "lj":
+                    s.set_lj(1.0, 1.0, 2.5, True, a, b)
+                else:
+                    s.set_lj_capped(1.0, 1.0, 2.5, 0.9, True, a, b)
+        if le:
+            s.set_lees_edwards(True, 0.1, 0.4)
+        s.set_thermostat(espp.ESPP_THERMO_DPD, 1.1)
+        s.set_state(np.concatenate([x for x, _ in group]), np.concatenate([v for _, v in group]), None)
+        s.build_neighbors(2.5, 0.3)
+        s.integrate(12, 0.004, 4.5, 0.72)
+        out.append(s.get_state())
+        s.close()
+    for a, b, both in zip(*out):
+        assert np.array_equal(np.concatenate([a, b]), both)
